@@ -283,9 +283,9 @@ gpr_status ppr_target(const gpr_graph* g, int32_t target, double damping, double
  *   x_0 = e_s;  x_{k+1}[v] = (1 - d) e_s[v] + d (sum_{u->v} x_k[u]/outdeg(u) + D_k e_s[v])
  * A column stops after max_iters steps, or, if tol > 0, after the first step
  * k with d/(1-d) * ||x_k - x_{k-1}||_1 <= tol (an a-posteriori bound on the
- * L1 distance to the fixed point).  One call runs every column of every job
- * in one persistent launch; a column's result does not depend on the other
- * columns or jobs in the call. */
+ * L1 distance to the fixed point).  One call runs every column of every job;
+ * a column's result does not depend on the other columns or jobs in the
+ * call. */
 typedef struct {
   const gpr_graph* graph;
   int32_t num_seeds;     /* K >= 1 columns */
@@ -306,24 +306,25 @@ gpr_status ppr_batch(const gpr_ppr_job* jobs, int32_t num_jobs, int32_t max_iter
 
 /* ---- autotuner for the batched launch (no counterpart in the paper) -------
  * ppr_batch groups its 64-column jobs by graph size, class k holding graphs
- * with ceil(log2 n) <= log2n_max[k] (11, 13, 15, 17, then all larger), and
- * runs each class as one persistent launch of thread-block clusters, each
- * cluster one job at a time, its rows split among the cluster's CTAs.  The
- * CTAs per cluster (1, 2, 4 or 8) of a (class, dt): ppr_tune times each on
- * up to 64 of the class's jobs in `jobs` (trial_steps in [1, 1000] steps per
- * trial; the jobs' outputs are overwritten) and keeps the fastest for later
- * ppr_batch calls in this process; a class never tuned takes 4 CTAs (8 for
- * ceil log2 n in 14..15, the choice measured on GB300 for R-MAT graphs).  The
- * environment variable GPR_PPR_CLUSTER=1|2|4|8 forces one shape for every
- * class.  A column's bits depend on its class's shape (the row split orders
- * the FP64 partial sums), never on the other columns or jobs of a call.
+ * with ceil(log2 n) <= log2n_max[k] (11, 13, 15, 17, then all larger).  A
+ * class runs either step by step, each step of all of its jobs spread over
+ * the whole GPU, or as one persistent launch of thread-block clusters, each
+ * cluster one job at a time, its rows split among the cluster's CTAs.
+ * ppr_tune times 1, 2, 4 and 8 CTAs per cluster and the step-by-step
+ * schedule for each (class, dt) on up to 64 of the class's jobs in `jobs`
+ * (trial_steps in [1, 1000] steps per trial; the jobs' outputs are
+ * overwritten) and keeps the fastest for later ppr_batch calls in this
+ * process; a class never tuned runs step by step.  The environment variable
+ * GPR_PPR_CLUSTER=1|2|4|8 forces one cluster shape for every class.  A
+ * column's bits depend on its class's schedule (the order of its sums),
+ * never on the other columns or jobs of a call.
  * Synchronous.  out may be NULL. */
 typedef struct {
   int32_t classes;         /* classes present in the jobs (entries below) */
   int32_t log2n_max[5];    /* the class's largest ceil(log2 n) (31: unbounded) */
   int32_t jobs[5];         /* 64-column jobs of the class */
-  int32_t cluster[5];      /* CTAs per cluster chosen */
-  double ms[5];            /* trial time with the chosen shape */
+  int32_t cluster[5];      /* CTAs per cluster of the fastest cluster shape */
+  double ms[5];            /* trial time with that shape */
   double ms_cluster8[5];   /* trial time with 8 CTAs per cluster */
 } gpr_ppr_tune_result;
 

@@ -11,8 +11,9 @@
 // lane.  Rows longer than one warp's fair share are handled by the whole
 // block with a fixed-order combine.
 //
-// ppr_batch: each job runs on one thread-block cluster for all of its steps,
-// in a per-cluster workspace.  The
+// ppr_batch runs its jobs step by step over the whole GPU (ppr_steps.cu), or, a
+// class of graph sizes that ppr_tune found faster so, here: each job on one
+// thread-block cluster for all of its steps, in a per-cluster workspace.  The
 // cluster's blocks split the rows by edge count; after each step they meet at
 // the hardware cluster barrier, then every block folds the per-column FP64
 // partials of all blocks (read through distributed shared memory) in rank
@@ -822,6 +823,25 @@ __global__ void part_bounds_kernel(const int32_t* __restrict__ col_ptr, int32_t 
 
 // ---- host side ----------------------------------------------------------------
 
+void heavy_of(const gpr_graph* g, const int32_t** rows, int32_t* n, int32_t* deg, int32_t* split0) {
+  const Plan& P = g->plan;
+  *rows = P.rows;
+  *n = 0;
+  *deg = INT_MAX;
+  *split0 = 0;
+  // the long rows are the last chunked (lanes 0) bucket; the plan's split
+  // entries list the rows of every chunked bucket in bucket order
+  int32_t before = 0;
+  for (int b = 0; b < P.nbuckets; ++b)
+    if (P.bucket[b].lanes == 0) {
+      *split0 = before;
+      *rows = P.rows + P.bucket[b].row_begin;
+      *n = P.bucket[b].row_end - P.bucket[b].row_begin;
+      *deg = b > 0 ? P.deg_threshold[b - 1] : -1;  // bucket 0 holds every degree from 0
+      before += *n;
+    }
+}
+
 template <typename T>
 static int max_clusters_for(int cluster) {
   cudaLaunchConfig_t cfg = {};
@@ -926,18 +946,21 @@ static void ppr_launch(PprJob* jobs_dev, const int32_t* order_dev, int32_t njobs
 
 // ---- graph-size classes and the cluster-shape autotuner ---------------------
 // A job's graph falls in class k by ceil(log2 n): <= 11, 12-13, 14-15, 16-17,
-// >= 18.  Each class present in a call runs as its own persistent launch with
-// its own number of CTAs per cluster: one CTA suits a small graph (its steps
-// need no cluster barrier and its rows fill one CTA), eight a large one.
-// ppr_tune times the shapes of a (class, storage type) on a sample of the
-// class's jobs and keeps the fastest for the process; an untuned class takes
-// kDefaultShape.  A column's bits depend on its class's shape (the row split
-// among a cluster's CTAs orders the FP64 partial sums), not on the other
-// columns or jobs of the call.
+// >= 18.  A class runs step by step over the whole GPU (ppr_steps.cu) or as
+// its own persistent launch with its own number of CTAs per cluster.
+// ppr_tune times the cluster shapes and the step-major schedule of a (class,
+// storage type) on a sample of the class's jobs and keeps the fastest for the
+// process; an untuned class is step-major: measured faster for every class on
+// R-MAT batches (256 graphs of 1,000 to 2,000 nodes, the smallest class, are
+// even: 15.8 ms against 15.7 with two CTAs per cluster; a single such graph
+// with one seed takes 1.0 ms against 2.0 to 3.7).  A column's bits depend on
+// its class's schedule (the order of its sums), not on the other columns or
+// jobs of the call.
 constexpr int kPprClasses = 5;
 constexpr int kClusterCands[] = {1, 2, 4, 8};
 constexpr int kDefaultCluster = 8;
-constexpr int kDefaultShape[kPprClasses] = {4, 4, 8, 4, 4};  // measured on GB300 (R-MAT batch, FP32 and BF16)
+constexpr int kStepMajor = 0;  // a class's "shape" when its jobs run step by step over the whole GPU (ppr_steps.cu)
+constexpr int kDefaultShape[kPprClasses] = {kStepMajor, kStepMajor, kStepMajor, kStepMajor, kStepMajor};
 constexpr int32_t kTuneSampleJobs = 64;
 constexpr int64_t kWorkspaceBudget = (int64_t)16 << 30;  // per launch: clusters x stride at most
 
@@ -993,8 +1016,8 @@ static void launch_set(PprJob* jobs_dev, const std::vector<int32_t>& order, int3
 // the call's real run then overwrites.
 template <typename A>
 static int tune_class(const std::vector<PprJob>& dj, const std::vector<std::vector<PprCol>>& cols,
-                      const std::vector<int32_t>& members, int32_t n_cap, gpr_dtype dt, int32_t trial_steps,
-                      cudaStream_t s, A alloc, double* ms_out) {
+                      const std::vector<StepRequest>& reqs, const std::vector<int32_t>& members, int32_t n_cap,
+                      gpr_dtype dt, int32_t trial_steps, cudaStream_t s, A alloc, double* ms_out, bool* step_major) {
   std::vector<int32_t> pick;
   const int32_t step = std::max<int32_t>(1, (int32_t)members.size() / kTuneSampleJobs);
   for (size_t i = 0; i < members.size() && (int32_t)pick.size() < kTuneSampleJobs; i += step) pick.push_back(members[i]);
@@ -1017,22 +1040,34 @@ static int tune_class(const std::vector<PprJob>& dj, const std::vector<std::vect
   GPR_CUDA(cudaMemcpyAsync(tjobs, tj.data(), (size_t)nt * sizeof(PprJob), cudaMemcpyHostToDevice, s));
   std::vector<int32_t> order(nt);
   std::iota(order.begin(), order.end(), 0);
+  std::vector<StepRequest> treqs(nt);
+  for (int32_t i = 0; i < nt; ++i) {
+    treqs[i] = reqs[pick[i]];
+    treqs[i].cols = tcols + (size_t)i * kPprCols;
+  }
   cudaEvent_t e0 = nullptr, e1 = nullptr;
   GPR_CUDA(cudaEventCreate(&e0));
   GPR_CUDA(cudaEventCreate(&e1));
   int best = kDefaultCluster;
   float best_ms = 0.f;
   try {
-    for (int ci = 0; ci < 4; ++ci) {
-      const int cl = kClusterCands[ci];
+    for (int ci = 0; ci < 5; ++ci) {  // the cluster shapes, then the step-major schedule
+      const int cl = ci < 4 ? kClusterCands[ci] : kStepMajor;
       float ms = 0.f;
       for (int rep = 0; rep < 2; ++rep) {  // the first run warms the caches
         GPR_CUDA(cudaMemcpyAsync(tcols, flat.data(), flat.size() * sizeof(PprCol), cudaMemcpyHostToDevice, s));
         GPR_CUDA(cudaEventRecord(e0, s));
-        launch_set(tjobs, order, n_cap, dt, cl, s, alloc);
+        if (cl == kStepMajor)
+          run_ppr_steps(treqs, trial_steps, false, dt, s);
+        else
+          launch_set(tjobs, order, n_cap, dt, cl, s, alloc);
         GPR_CUDA(cudaEventRecord(e1, s));
         GPR_CUDA(cudaStreamSynchronize(s));
         GPR_CUDA(cudaEventElapsedTime(&ms, e0, e1));
+      }
+      if (cl == kStepMajor) {
+        *step_major = ms < best_ms;
+        break;
       }
       ms_out[ci] = ms;
       if (ci == 0 || ms < best_ms) {
@@ -1074,15 +1109,8 @@ static gpr_status run_ppr(const gpr_ppr_job* jobs, int32_t num_jobs, int32_t max
         J.n = g->n;
         J.col_ptr = g->col_ptr;
         J.row_idx = g->row_idx;
-        J.heavy_rows = g->plan.rows;
-        J.n_heavy = 0;
-        J.heavy_deg = INT_MAX;
-        for (int b = 0; b < g->plan.nbuckets; ++b)
-          if (g->plan.bucket[b].lanes == 0) {
-            J.heavy_rows = g->plan.rows + g->plan.bucket[b].row_begin;
-            J.n_heavy = g->plan.bucket[b].row_end - g->plan.bucket[b].row_begin;
-            J.heavy_deg = b > 0 ? g->plan.deg_threshold[b - 1] : -1;  // bucket 0 holds every degree from 0
-          }
+        int32_t split0 = 0;
+        heavy_of(g, &J.heavy_rows, &J.n_heavy, &J.heavy_deg, &split0);
         J.iters = max_iters;
         std::vector<PprCol> cc(kPprCols);
         for (int k = 0; k < kPprCols; ++k) {
@@ -1134,7 +1162,12 @@ static gpr_status run_ppr(const gpr_ppr_job* jobs, int32_t num_jobs, int32_t max
     std::vector<PprCol> flat((size_t)nj * kPprCols);
     for (int32_t i = 0; i < nj; ++i)
       std::copy(cols[i].begin(), cols[i].end(), flat.begin() + (size_t)i * kPprCols);
-    for (int32_t i = 0; i < nj; ++i) dj[i].cols = cols_dev + (size_t)i * kPprCols;
+    std::vector<StepRequest> reqs(nj);
+    for (int32_t i = 0; i < nj; ++i) {
+      dj[i].cols = cols_dev + (size_t)i * kPprCols;
+      const gpr_ppr_job& rq = jobs[src[i].first];
+      reqs[i] = StepRequest{rq.graph, std::min(rq.num_seeds - src[i].second, kPprCols), dj[i].cols};
+    }
     PprJob* jobs_dev = (PprJob*)T((size_t)nj * sizeof(PprJob));
     GPR_CUDA(cudaMemcpyAsync(jobs_dev, dj.data(), (size_t)nj * sizeof(PprJob), cudaMemcpyHostToDevice, s));
     // the shape of each class
@@ -1151,10 +1184,11 @@ static gpr_status run_ppr(const gpr_ppr_job* jobs, int32_t num_jobs, int32_t max
       }
       if (tune_all) {
         double ms[4] = {0, 0, 0, 0};
-        shape[k] = tune_class(dj, cols, members[k], ncap[k], dt, std::max(1, trial_steps), s, T, ms);
+        bool step_major = false;
+        shape[k] = tune_class(dj, cols, reqs, members[k], ncap[k], dt, std::max(1, trial_steps), s, T, ms, &step_major);
         {
           std::lock_guard<std::mutex> lk(g_ppr_tune_mu);
-          g_ppr_tuned[key] = shape[k];
+          g_ppr_tuned[key] = step_major ? kStepMajor : shape[k];
         }
         if (tres) {
           const int c = tres->classes++;
@@ -1175,7 +1209,14 @@ static gpr_status run_ppr(const gpr_ppr_job* jobs, int32_t num_jobs, int32_t max
       return GPR_OK;
     }
     GPR_CUDA(cudaMemcpyAsync(cols_dev, flat.data(), flat.size() * sizeof(PprCol), cudaMemcpyHostToDevice, s));
-    for (int k = 0; k < kPprClasses; ++k) launch_set(jobs_dev, members[k], ncap[k], dt, shape[k], s, T);
+    std::vector<StepRequest> stepped;
+    for (int k = 0; k < kPprClasses; ++k) {
+      if (shape[k] != kStepMajor)
+        launch_set(jobs_dev, members[k], ncap[k], dt, shape[k], s, T);
+      else
+        for (int32_t i : members[k]) stepped.push_back(reqs[i]);
+    }
+    run_ppr_steps(stepped, max_iters, tol > 0.0, dt, s);
     // per-column results back to the caller
     GPR_CUDA(cudaMemcpyAsync(flat.data(), cols_dev, flat.size() * sizeof(PprCol), cudaMemcpyDeviceToHost, s));
     GPR_CUDA(cudaStreamSynchronize(s));

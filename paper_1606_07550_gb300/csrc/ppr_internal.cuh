@@ -6,6 +6,10 @@
 #include <cuda_runtime.h>
 #include <stdint.h>
 
+#include <vector>
+
+#include "gpr_internal.cuh"
+
 namespace gpr {
 
 constexpr int kPprCols = 64;  // columns per job: 32 lanes x 2
@@ -110,5 +114,21 @@ void ppr_chunk_launch(const SlotDesc* slots_dev, const StepItem* items_dev, int3
 void ppr_part_bounds(const int32_t* col_ptr, int32_t n, int64_t m, int32_t nparts, int32_t* part_rows,
                      cudaStream_t s);
 
+// The long rows of g's plan (in-degree above *deg): *n ascending row ids, the
+// first of them split entry *split0 of the plan's chunk lists.
+void heavy_of(const gpr_graph* g, const int32_t** rows, int32_t* n, int32_t* deg, int32_t* split0);
+
+// ---- step-major execution of a batch (ppr_steps.cu) ------------------------
+// One graph with k <= 64 columns, whose 64 records are in device memory: the
+// outputs of columns 0..k-1 are consecutive floats of a row of x_out.
+struct StepRequest {
+  const gpr_graph* graph;
+  int32_t k;
+  PprCol* cols;
+};
+// Runs every request to its end on s (no synchronisation, but for every few
+// steps' look at the stops when tol) and leaves status, iters and residual in
+// the records.
+void run_ppr_steps(const std::vector<StepRequest>& reqs, int32_t max_iters, bool tol, gpr_dtype dt, cudaStream_t s);
 
 }  // namespace gpr

@@ -135,20 +135,7 @@ static void fill_desc(SlotDesc& D, const gpr_graph* g, const Slot* sl) {
   D.old2new = g->plan.old2new;
   D.new2old = g->plan.new2old;
   D.n = g->n;
-  D.heavy_rows = g->plan.rows;
-  D.n_heavy = 0;
-  D.heavy_deg = INT_MAX;
-  // the long rows are the last chunked (lanes 0) bucket; the plan's split
-  // entries list the rows of every chunked bucket in bucket order
-  int32_t before = 0;
-  for (int b = 0; b < g->plan.nbuckets; ++b)
-    if (g->plan.bucket[b].lanes == 0) {
-      D.heavy_split0 = before;
-      D.heavy_rows = g->plan.rows + g->plan.bucket[b].row_begin;
-      D.n_heavy = g->plan.bucket[b].row_end - g->plan.bucket[b].row_begin;
-      D.heavy_deg = b > 0 ? g->plan.deg_threshold[b - 1] : -1;  // bucket 0 holds every degree from 0
-      before += D.n_heavy;
-    }
+  heavy_of(g, &D.heavy_rows, &D.n_heavy, &D.heavy_deg, &D.heavy_split0);
   D.chunk_begin = g->plan.chunk_begin;
   D.chunk_end = g->plan.chunk_end;
   D.split_hbeg = g->plan.split_hbeg;
