@@ -22,7 +22,9 @@
 // kernel.  The bucket kernels of a step are independent and run as parallel
 // branches of one CUDA graph that holds the whole iteration loop.
 #include <algorithm>
+#include <functional>
 #include <map>
+#include <queue>
 #include <tuple>
 #include <vector>
 #include <chrono>
@@ -31,6 +33,7 @@
 #include <cstring>
 
 #include "blocked.cuh"
+#include "pr_persist.cuh"
 #include "pr_step.cuh"
 
 namespace gpr {
@@ -328,6 +331,20 @@ struct PagerankWork {
   int exec_sched = -1;
   bool exec_warm = false;
   int64_t exec_kernels = 0;  // kernel nodes in `exec`
+  // the single-launch iteration of small graphs (pr_persist.cuh)
+  bool pers = false;         // its layout is made
+  int32_t* pers_row = nullptr;
+  float* pers_inv = nullptr;
+  int2* pers_span = nullptr;
+  int32_t* pers_off = nullptr;
+  int32_t* pers_sell = nullptr;
+  int32_t* pers_deal = nullptr;
+  int pers_blocks = 0;
+  bool pers_cluster = false;
+  float* pers_x = nullptr;
+  int32_t pers_long = 0, pers_slices = 0;
+  char* ctl = nullptr;       // barrier words (16 bytes), last log row (32), step sums
+  size_t ctl_cap = 0;
 };
 
 void pagerank_work_free(PagerankWork* w) {
@@ -348,6 +365,14 @@ void pagerank_work_free(PagerankWork* w) {
   dfree(w->prm, s);
   dfree(w->arrive, s);
   dfree(w->log, s);
+  dfree(w->pers_row, s);
+  dfree(w->pers_inv, s);
+  dfree(w->pers_span, s);
+  dfree(w->pers_off, s);
+  dfree(w->pers_sell, s);
+  dfree(w->pers_deal, s);
+  dfree(w->pers_x, s);
+  dfree(w->ctl, s);
   if (w->ev_fork) cudaEventDestroy(w->ev_fork);
   if (w->ev_t0) cudaEventDestroy(w->ev_t0);
   if (w->ev_t1) cudaEventDestroy(w->ev_t1);
@@ -742,6 +767,266 @@ static Choice pick(gpr_graph* g, PagerankWork* w, int flags, gpr_dtype dt, cudaS
   return Choice{};
 }
 
+// ---- the iteration of a small graph in one launch (pr_persist.cuh) ------------
+
+// Whether the call takes it: the pull schedule of a graph below kTuneMinEdges
+// from the uniform vector, without the hot pass.  (A warm start's vector need
+// not sum to about one, as the kernel's fixed-point sums want it.)
+static bool persist_eligible(const gpr_graph* g, const PagerankWork* w, int sched, bool warm) {
+  // a block's long rows fit its lists: at most m / 65 rows, dealt out evenly
+  static_assert(kTuneMinEdges / (kPersShort + 1) / 128 < kPersLongRows, "long rows of a block");
+  return sched == kSchedPull && !warm && w->hot_grid == 0 && g->m < kTuneMinEdges && num_sms() >= 128;
+}
+
+// Contributions kept in shared memory, in bytes: all of a graph's, or the
+// most-read ones.  32 to 128 KB measured within 2% of each other at 250,000
+// nodes and 4,000,000 edges (200 KB takes 10% longer to fill than it saves,
+// none takes twice as long).
+constexpr int32_t kPersHotBytes = 64 << 10;
+
+// Graphs of up to this much work (edges + 4 * rows) run on one cluster, whose
+// barrier is faster: 1,000 nodes and 5,000 edges 2.9 us a step against 3.3 over
+// all SMs; 10,000 and 100,000 even; 20,000 and 200,000 (R-MAT) 10.6 against 6.3.
+constexpr int64_t kPersClusterWork = 1 << 16;
+constexpr int kPersClusterBlocks = 16;
+
+// Whether a cluster of that many blocks of the kernel fits on this GPU.
+static bool persist_cluster_fits(int blocks) {
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3((unsigned)blocks, 1, 1);
+  cfg.blockDim = dim3(kPersThreads, 1, 1);
+  cfg.dynamicSmemBytes = kPersHotBytes;
+  cudaLaunchAttribute attr[1];
+  attr[0].id = cudaLaunchAttributeClusterDimension;
+  attr[0].val.clusterDim.x = (unsigned)blocks;
+  attr[0].val.clusterDim.y = 1;
+  attr[0].val.clusterDim.z = 1;
+  cfg.attrs = attr;
+  cfg.numAttrs = 1;
+  int num = 0;
+  const bool ok =
+      cudaFuncSetAttribute(persist_kernel<float, true>, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) ==
+          cudaSuccess &&
+      cudaFuncSetAttribute(persist_kernel<float, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, kPersHotBytes) ==
+          cudaSuccess &&
+      cudaOccupancyMaxActiveClusters(&num, persist_kernel<float, true>, &cfg) == cudaSuccess && num > 0;
+  cudaGetLastError();
+  return ok;
+}
+
+// Deals the long rows (edges[]) and the slices (off[]) to nblk blocks by
+// estimated cycles, the largest first, to the block with the least so far (see
+// PersistArgs::deal).  A block's lists in shared memory hold kPersLongRows rows
+// and kPersChunks chunks.
+static std::vector<int32_t> persist_deal(const std::vector<int2>& edges, const std::vector<int32_t>& off, int nblk) {
+  using Load = std::pair<int64_t, int>;
+  std::priority_queue<Load, std::vector<Load>, std::greater<Load>> heap;
+  std::vector<std::vector<int32_t>> rows(nblk), slices(nblk);
+  std::vector<int64_t> load(nblk, 0);
+  std::vector<int32_t> chunks(nblk, 0);
+  for (int b = 0; b < nblk; ++b) heap.push(Load(0, b));
+  for (size_t i = 0; i < edges.size(); ++i) {  // by descending in-degree
+    const int32_t deg = edges[i].y - edges[i].x, c = pers_chunk(deg), k = (deg + c - 1) / c;
+    while (!heap.empty()) {
+      const int b = heap.top().second;
+      heap.pop();
+      if ((int)rows[b].size() >= kPersLongRows || chunks[b] + k > kPersChunks) continue;  // full
+      rows[b].push_back((int32_t)i);
+      chunks[b] += k;
+      load[b] += deg / 3 + 60 * k;
+      heap.push(Load(load[b], b));
+      break;
+    }
+  }
+  heap = {};
+  for (int b = 0; b < nblk; ++b) heap.push(Load(load[b], b));
+  const int32_t ns = (int32_t)off.size() - 1, bundle = std::max(1, ns / 8192);
+  for (int32_t s = 0; s < ns; s += bundle) {
+    const int b = heap.top().second;
+    heap.pop();
+    for (int32_t t = s; t < std::min(ns, s + bundle); ++t) {
+      slices[b].push_back(t);
+      load[b] += (off[t + 1] - off[t]) / 3 + 150;
+    }
+    heap.push(Load(load[b], b));
+  }
+  std::vector<int32_t> deal((size_t)2 * nblk + 2);
+  for (int b = 0; b < nblk; ++b) {
+    deal[b] = (int32_t)deal.size();
+    deal.insert(deal.end(), rows[b].begin(), rows[b].end());
+  }
+  deal[nblk] = (int32_t)deal.size();
+  for (int b = 0; b < nblk; ++b) {
+    deal[nblk + 1 + b] = (int32_t)deal.size();
+    deal.insert(deal.end(), slices[b].begin(), slices[b].end());
+  }
+  deal[2 * nblk + 1] = (int32_t)deal.size();
+  return deal;
+}
+
+static void persist_layout(gpr_graph* g, PagerankWork* w, cudaStream_t s) {
+  const Plan& P = g->plan;
+  const int32_t n = g->n;
+  const int b = g->id_bits;
+  int* derr = nullptr;
+  int32_t* count = nullptr;
+  uint64_t *keys = nullptr, *alt = nullptr;
+  auto release = [&]() {
+    dfree(derr, s);
+    dfree(count, s);
+    dfree(keys, s);
+    dfree(alt, s);
+  };
+  try {
+    derr = (int*)dalloc(16, s);
+    count = (int32_t*)dalloc((kPersShort + 2) * 4, s);
+    keys = (uint64_t*)dalloc((size_t)n * 8, s);
+    alt = (uint64_t*)dalloc((size_t)n * 8, s);
+    GPR_CUDA(cudaMemsetAsync(derr, 0, 16, s));
+    GPR_CUDA(cudaMemsetAsync(count, 0, (kPersShort + 2) * 4, s));
+    const int grid = (int)std::min<int64_t>(((int64_t)n + 255) / 256, num_sms() * 8);
+    persist_keys_kernel<<<grid, 256, 0, s>>>(g->col_ptr, n, b, g->max_in, keys, count);
+    GPR_CUDA(cudaGetLastError());
+    int32_t h[kPersShort + 2];
+    GPR_CUDA(cudaMemcpyAsync(h, count, sizeof h, cudaMemcpyDeviceToHost, s));
+    const uint64_t* sorted = radix_sort_u64(keys, alt, n, b + ceil_log2((int64_t)g->max_in + 1), s, derr);
+    GPR_CUDA(cudaStreamSynchronize(s));
+    // slice widths: the in-degree of a slice's first row
+    w->pers_long = h[kPersShort + 1];
+    const int32_t ns = (n - w->pers_long + 31) / 32;
+    w->pers_slices = ns;
+    std::vector<int32_t> off((size_t)ns + 1, 0);
+    int deg = kPersShort;
+    int64_t rows = 0;  // sliced rows of more than `deg - 1` edges
+    rows += h[deg];
+    for (int32_t k = 0; k < ns; ++k) {
+      while (rows <= (int64_t)32 * k && deg > 0) rows += h[--deg];
+      off[k + 1] = off[k] + 32 * deg;
+    }
+    w->pers_row = (int32_t*)dalloc((size_t)n * 4, s);
+    w->pers_inv = (float*)dalloc((size_t)n * 4, s);
+    w->pers_span = (int2*)dalloc((size_t)std::max(w->pers_long, 1) * 8, s);
+    w->pers_off = (int32_t*)dalloc(off.size() * 4, s);
+    w->pers_sell = (int32_t*)dalloc((size_t)std::max(off[ns], 1) * 4, s);
+    w->pers_x = (float*)dalloc((size_t)n * 4, s);
+    GPR_CUDA(cudaMemcpyAsync(w->pers_off, off.data(), off.size() * 4, cudaMemcpyHostToDevice, s));
+    persist_layout_kernel<<<grid, 256, 0, s>>>(sorted, b, g->col_ptr, g->row_idx, P.inv_deg, n, w->pers_long, ns,
+                                              w->pers_off, w->pers_row, w->pers_inv, w->pers_span, w->pers_sell);
+    GPR_CUDA(cudaGetLastError());
+    count_launches(2);
+    int bad = 0;
+    std::vector<int2> edges(w->pers_long);
+    GPR_CUDA(cudaMemcpyAsync(&bad, derr, 4, cudaMemcpyDeviceToHost, s));
+    if (w->pers_long > 0)
+      GPR_CUDA(cudaMemcpyAsync(edges.data(), w->pers_span, edges.size() * 8, cudaMemcpyDeviceToHost, s));
+    GPR_CUDA(cudaStreamSynchronize(s));
+    if (bad & DERR_TIMEOUT) throw StatusFail{GPR_ETIMEOUT, "a look-back wait gave up"};
+    w->pers_cluster = g->m + 4 * (int64_t)n <= kPersClusterWork && persist_cluster_fits(kPersClusterBlocks);
+    w->pers_blocks = w->pers_cluster ? kPersClusterBlocks : num_sms();
+    const std::vector<int32_t> deal = persist_deal(edges, off, w->pers_blocks);
+    if (deal.size() != (size_t)(2 * w->pers_blocks + 2 + w->pers_long + ns))
+      throw StatusFail{GPR_EINVAL, "the long rows do not fit the blocks"};
+    w->pers_deal = (int32_t*)dalloc(deal.size() * 4, s);
+    GPR_CUDA(cudaMemcpyAsync(w->pers_deal, deal.data(), deal.size() * 4, cudaMemcpyHostToDevice, s));
+    release();
+    w->pers = true;
+  } catch (...) {
+    release();
+    for (void* p : {(void*)w->pers_row, (void*)w->pers_inv, (void*)w->pers_span, (void*)w->pers_off,
+                    (void*)w->pers_sell, (void*)w->pers_deal, (void*)w->pers_x})
+      dfree(p, s);
+    w->pers_row = w->pers_off = w->pers_sell = w->pers_deal = nullptr;
+    w->pers_inv = w->pers_x = nullptr;
+    w->pers_span = nullptr;
+    throw;
+  }
+}
+
+template <typename T, bool kCluster>
+static void launch_persist(const PersistArgs& A, int blocks, size_t smem, cudaStream_t s) {
+  GPR_CUDA(cudaFuncSetAttribute(persist_kernel<T, kCluster>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3((unsigned)blocks, 1, 1);
+  cfg.blockDim = dim3(kPersThreads, 1, 1);
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = s;
+  cudaLaunchAttribute attr[1];
+  if (kCluster) {
+    GPR_CUDA(cudaFuncSetAttribute(persist_kernel<T, kCluster>, cudaFuncAttributeNonPortableClusterSizeAllowed, 1));
+    attr[0].id = cudaLaunchAttributeClusterDimension;
+    attr[0].val.clusterDim.x = (unsigned)blocks;
+    attr[0].val.clusterDim.y = 1;
+    attr[0].val.clusterDim.z = 1;
+  } else {
+    attr[0].id = cudaLaunchAttributeCooperative;
+    attr[0].val.cooperative = 1;
+  }
+  cfg.attrs = attr;
+  cfg.numAttrs = 1;
+  GPR_CUDA(cudaLaunchKernelEx(&cfg, persist_kernel<T, kCluster>, A));
+  count_launches(1);
+}
+
+template <typename T>
+static void run_persist(gpr_graph* g, PagerankWork* w, double damping, int32_t iters, float* dst, cudaStream_t s) {
+  const Plan& P = g->plan;
+  const int32_t n = g->n;
+  const size_t need = 48 + ((size_t)iters + 1) * 24;
+  if (w->ctl_cap < need) {
+    dfree(w->ctl, s);
+    w->ctl = nullptr;
+    w->ctl_cap = 0;
+    const size_t cap = std::max<size_t>(need, 4096);
+    w->ctl = (char*)dalloc(cap, s);
+    w->ctl_cap = cap;
+  }
+  GPR_CUDA(cudaMemsetAsync(w->ctl, 0, need, s));
+  PersistArgs A{};
+  A.row_idx = g->row_idx;
+  A.row = w->pers_row;
+  A.inv = w->pers_inv;
+  A.span = w->pers_span;
+  A.off = w->pers_off;
+  A.sell = w->pers_sell;
+  A.deal = w->pers_deal;
+  A.n_long = w->pers_long;
+  A.nslices = w->pers_slices;
+  A.inv_deg = P.inv_deg;
+  A.old2new = P.old2new;
+  A.n = n;
+  A.H = std::min<int32_t>(n, kPersHotBytes / (int)sizeof(T)) & ~7;
+  A.xi = w->pers_x;
+  A.x = w->x[0];
+  A.c[0] = w->c[0];
+  A.c[1] = w->c[1];
+  A.bar = (unsigned int*)w->ctl;
+  A.log_row = (double*)(w->ctl + 16);
+  A.sums = (unsigned long long*)(w->ctl + 48);
+  A.out = dst;
+  auto split = [](double v, float* hi, float* lo) {
+    *hi = (float)v;
+    *lo = (float)(v - (double)*hi);
+  };
+  split(damping, &A.d_hi, &A.d_lo);
+  split((1.0 - damping) / (double)n, &A.t_hi, &A.t_lo);
+  split(1.0 / (double)n, &A.in_hi, &A.in_lo);
+  A.iters = iters;
+  const size_t smem = std::max<size_t>((size_t)A.H * sizeof(T), 16);
+  if (w->pers_cluster)
+    launch_persist<T, true>(A, w->pers_blocks, smem, s);
+  else
+    launch_persist<T, false>(A, w->pers_blocks, smem, s);
+}
+
+// Whether the launch's barrier gave up (a call that does not synchronise sees
+// NaN ranks instead).
+static void check_persist(PagerankWork* w, cudaStream_t s) {
+  unsigned int bad = 0;
+  GPR_CUDA(cudaMemcpyAsync(&bad, w->ctl + 4, 4, cudaMemcpyDeviceToHost, s));
+  GPR_CUDA(cudaStreamSynchronize(s));
+  if (bad) throw StatusFail{GPR_ETIMEOUT, "a block waited too long for the others"};
+}
+
 gpr_status run_pagerank(gpr_graph* g, double damping, int32_t iters, gpr_dtype dt, int flags, float* x_out,
                         gpr_stats* st, cudaStream_t s) {
   std::lock_guard<std::mutex> lock(g->mu);
@@ -770,31 +1055,49 @@ gpr_status run_pagerank(gpr_graph* g, double damping, int32_t iters, gpr_dtype d
       GPR_CUDA(cudaGetLastError());
       count_launches(1);
     }
-    ensure_exec(g, w, iters, dt, sched, warm, s);
-    StepParams hp{0.f, 0.f, damping, (double)g->n};
-    GPR_CUDA(cudaMemcpyAsync(w->prm, &hp, sizeof hp, cudaMemcpyHostToDevice, s));
-    const double t_setup =
-        std::chrono::duration<double, std::milli>(std::chrono::steady_clock::now() - t_setup0).count();
-    if (st) GPR_CUDA(cudaEventRecord(w->ev_t0, s));
-    GPR_CUDA(cudaGraphLaunch(w->exec, s));
-    if (st) GPR_CUDA(cudaEventRecord(w->ev_t1, s));
-    count_launches(w->exec_kernels);
-    const float* xf = w->x[iters & 1];
+    const bool persist = persist_eligible(g, w, sched, warm);
+    if (persist) {
+      // (a stream being captured cannot take the graph launch of the other way either)
+      cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+      GPR_CUDA(cudaStreamIsCapturing(s, &cap));
+      if (cap != cudaStreamCaptureStatusNone) throw CudaFail{cudaErrorStreamCaptureUnsupported, "pagerank"};
+      if (!w->pers) persist_layout(g, w, s);
+    } else {
+      ensure_exec(g, w, iters, dt, sched, warm, s);
+      StepParams hp{0.f, 0.f, damping, (double)g->n};
+      GPR_CUDA(cudaMemcpyAsync(w->prm, &hp, sizeof hp, cudaMemcpyHostToDevice, s));
+    }
     float* dst = (flags & GPR_PTR_HOST) ? nullptr : x_out;
     if (!dst) {
       if (!w->out_tmp) w->out_tmp = (float*)dalloc((size_t)g->n * 4, s);
       dst = w->out_tmp;
     }
-    const int og = (int)std::max<int64_t>(1, std::min<int64_t>(((int64_t)g->n + 255) / 256, num_sms() * 8));
-    output_kernel<<<og, 256, 0, s>>>(xf, g->plan.old2new, g->n, dst);
-    GPR_CUDA(cudaGetLastError());
-    count_launches(1);
+    const double t_setup =
+        std::chrono::duration<double, std::milli>(std::chrono::steady_clock::now() - t_setup0).count();
+    if (st) GPR_CUDA(cudaEventRecord(w->ev_t0, s));
+    if (persist) {
+      if (dt == GPR_BF16)
+        run_persist<__nv_bfloat16>(g, w, damping, iters, dst, s);
+      else
+        run_persist<float>(g, w, damping, iters, dst, s);
+      if (st) GPR_CUDA(cudaEventRecord(w->ev_t1, s));
+    } else {
+      GPR_CUDA(cudaGraphLaunch(w->exec, s));
+      if (st) GPR_CUDA(cudaEventRecord(w->ev_t1, s));
+      count_launches(w->exec_kernels);
+      const int og = (int)std::max<int64_t>(1, std::min<int64_t>(((int64_t)g->n + 255) / 256, num_sms() * 8));
+      output_kernel<<<og, 256, 0, s>>>(w->x[iters & 1], g->plan.old2new, g->n, dst);
+      GPR_CUDA(cudaGetLastError());
+      count_launches(1);
+    }
     if (flags & GPR_PTR_HOST) {
       GPR_CUDA(cudaMemcpyAsync(x_out, dst, (size_t)g->n * 4, cudaMemcpyDeviceToHost, s));
     }
     if (st) {
       double row[3];
-      GPR_CUDA(cudaMemcpyAsync(row, w->log + 3 * (int64_t)iters, sizeof row, cudaMemcpyDeviceToHost, s));
+      const void* log_row = persist ? (const void*)(w->ctl + 16) : w->log + 3 * (int64_t)iters;
+      GPR_CUDA(cudaMemcpyAsync(row, log_row, sizeof row, cudaMemcpyDeviceToHost, s));
+      if (persist) check_persist(w, s);
       GPR_CUDA(cudaStreamSynchronize(s));
       st->iters_run = iters;
       st->mass = row[0];
@@ -806,6 +1109,7 @@ gpr_status run_pagerank(gpr_graph* g, double damping, int32_t iters, gpr_dtype d
       st->t_setup_ms = t_setup;
       st->schedule = sched == kSchedBlocked ? GPR_SPMV_BLOCKED : GPR_SPMV_PULL;
     } else if (flags & GPR_PTR_HOST) {
+      if (persist) check_persist(w, s);
       GPR_CUDA(cudaStreamSynchronize(s));
     }
     return GPR_OK;

@@ -1,0 +1,81 @@
+"""PageRank of small graphs in one launch: rows at the edges of its cases (slices
+of 32 rows, groups of 8 indices, long rows and their chunks), sizes on both
+sides of the cluster's limit, against the FP64 oracle and the pull schedule's
+kernels (which a warm start from the uniform vector takes)."""
+import numpy as np
+import pytest
+
+import oracle
+import paper_1606_07550_gb300 as gpr
+
+from gpu_util import l1
+
+pytestmark = pytest.mark.gpu
+
+
+def tolerance(dt, iters, d=0.85):
+    # BF16 rounds each contribution by at most 2^-9 of itself, so a step moves at
+    # most d 2^-9 of the mass (on a graph of a few nodes nothing averages out),
+    # and each later step shrinks that by d
+    return 1e-5 + (d * 2.0 ** -9 * (1 - d ** iters) / (1 - d) if dt == gpr.BF16 else 0.0)
+
+
+DEGREES = [0, 1, 7, 8, 9, 15, 16, 17, 63, 64, 65, 255, 256, 257, 511, 513, 4095, 16_385, 20_000]
+
+
+def star_rows(n, extra, rng):
+    """Rows of the in-degrees above, and `extra` random edges."""
+    src, dst = [], []
+    for i, deg in enumerate(d for d in DEGREES if d < n - 1):
+        v = (5 + 7 * i) % n
+        s = rng.choice(n - 1, deg, replace=False)
+        src.append(s + (s >= v))
+        dst.append(np.full(deg, v))
+    src.append(rng.integers(0, n, extra))
+    dst.append(rng.integers(0, n, extra))
+    return np.concatenate(src).astype(np.int32), np.concatenate(dst).astype(np.int32)
+
+
+def run(torch, g, iters, dt, warm=False, stats=False):
+    x = torch.full((g.n,), 1.0 / g.n, dtype=torch.float32, device="cuda")
+    st = gpr.pagerank(g, x, iters=iters, dtype=dt, warm_start=warm, stats=stats)
+    return x.cpu().numpy(), st
+
+
+@pytest.mark.parametrize("n,extra", [(1, 0), (2, 1), (31, 0), (33, 40), (1000, 5000), (16_000, 1000), (16_400, 0),
+                                     (25_000, 60_000), (70_001, 500_000)])
+@pytest.mark.parametrize("dt", [gpr.FP32, gpr.BF16])
+def test_sizes_and_row_lengths(n, extra, dt):
+    import torch
+    src, dst = star_rows(n, extra, np.random.default_rng(n))
+    g = gpr.graph_build(torch.from_numpy(src).cuda(), torch.from_numpy(dst).cuda(), n)
+    ref = oracle.build_csc(n, src, dst)
+    for iters in (0, 1, 2, 40):
+        x, st = run(torch, g, iters, dt, stats=True)
+        xr = oracle.pagerank(ref, 0.85, iters)
+        assert l1(x, xr) <= tolerance(dt, iters)
+        assert abs(st.mass - x.astype(np.float64).sum()) <= 1e-6
+        assert abs(st.dangling - x.astype(np.float64)[ref.outdeg == 0].sum()) <= 1e-6
+        # the general kernels, from the same start
+        y, sy = run(torch, g, iters, dt, warm=True, stats=True)
+        assert np.abs(x.astype(np.float64) - y).sum() <= 2 * tolerance(dt, iters)
+        assert abs(st.residual_l1 - sy.residual_l1) <= 2 * tolerance(dt, iters)
+        # the same bits again, with and without stats
+        assert (run(torch, g, iters, dt)[0] == x).all()
+
+
+def test_other_damping_and_two_graphs_in_turn():
+    import torch
+    rng = np.random.default_rng(8)
+    graphs = []
+    for n, m in ((300, 2000), (40_000, 300_000)):
+        src, dst = rng.integers(0, n, m).astype(np.int32), rng.integers(0, n, m).astype(np.int32)
+        graphs.append((gpr.graph_build(src, dst, n), oracle.build_csc(n, src, dst)))
+    for d in (0.5, 0.99):
+        outs = []
+        for g, _ in graphs * 2:  # nothing waits between the calls
+            x = torch.empty(g.n, dtype=torch.float32, device="cuda")
+            gpr.pagerank(g, x, damping=d, iters=30)
+            outs.append(x)
+        for (g, ref), x in zip(graphs * 2, outs):
+            assert l1(x.cpu().numpy(), oracle.pagerank(ref, d, 30)) <= 1e-5
