@@ -219,17 +219,16 @@ void blocked_free(Blocked* k, cudaStream_t s) {
 }
 
 template <typename K>
-static int persistent_grid(K kernel, size_t smem) {
+static int persistent_grid(K kernel, int threads, size_t smem) {
   GPR_CUDA(cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
   int per_sm = 0;
-  GPR_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kernel, kBkThreads, smem));
+  GPR_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kernel, threads, smem));
   return num_sms() * std::max(per_sm, 1);
 }
 
 Blocked* blocked_build(const gpr_graph* g, int sb_bits, int w_bits, int32_t n_dense_req, int64_t unit_edges,
                        cudaStream_t s) {
   const int64_t unit = std::max<int64_t>(unit_edges, 1 << 12);
-  const int64_t xunit = std::min<int64_t>(1 << 20, 4 * unit);  // expand units stage a source block each
   if (!blocked_eligible(g, sb_bits, w_bits))
     throw StatusFail{GPR_EINVAL, "the blocked schedule does not fit this graph"};
   Blocked* k = new Blocked();
@@ -328,6 +327,17 @@ Blocked* blocked_build(const gpr_graph* g, int sb_bits, int w_bits, int32_t n_de
     if (herr & DERR_TIMEOUT) throw StatusFail{GPR_ETIMEOUT, "blocked layout: a look-back wait of the sort timed out"};
     trace_phase("layout: extract + tables", s);
 
+    // Edges per expand unit: several units for every SM, so that no SM waits on
+    // a few large ones , but each worth staging its
+    // source block (128 KB) for.
+    int64_t other = m;
+    if (D < S) {
+      other = 0;
+      for (int32_t b = 0; b < B; ++b) other += X[(size_t)(S - 1) * B + b].y - X[(size_t)D * B + b].x;
+    }
+    const int64_t xunit =
+        std::max<int64_t>((int64_t)1 << 15, std::min<int64_t>((int64_t)1 << 20, other / ((int64_t)num_sms() * 4)));
+
     // expand units (source blocks past the dense ones): per source block,
     // runs of consecutive bins' segments of at most unit edges and
     // kMaxUnitSegs segments; a longer segment is cut into pieces of its own.
@@ -425,9 +435,9 @@ Blocked* blocked_build(const gpr_graph* g, int sb_bits, int w_bits, int32_t n_de
     k->ctr = (unsigned int*)dalloc(16, s);
     GPR_CUDA(cudaMemsetAsync(k->ctr, 0, 16, s));
     k->partials = (double*)dalloc((size_t)B * 3 * sizeof(double), s);
-    k->xgrid = persistent_grid(bk_expand_kernel, expand_smem(sb_bits));
-    k->agrid = std::max(persistent_grid(bk_accum_kernel<float>, accum_smem(w_bits)),
-                        persistent_grid(bk_accum_kernel<__nv_bfloat16>, accum_smem(w_bits)));
+    k->xgrid = persistent_grid(bk_expand_kernel, kBkThreads, expand_smem(sb_bits));
+    k->agrid = std::max(persistent_grid(bk_accum_kernel<float>, kBkThreads, accum_smem(w_bits)),
+                        persistent_grid(bk_accum_kernel<__nv_bfloat16>, kBkThreads, accum_smem(w_bits)));
     trace_phase("layout: upload", s);
     k->bytes = (int64_t)me * 8 + nseg * (int64_t)sizeof(int2) + (int64_t)xu.size() * sizeof(ExpandUnit) +
                (int64_t)au.size() * sizeof(AccumUnit) + (int64_t)n_split * (int64_t)W * 8 + (int64_t)B * 24;

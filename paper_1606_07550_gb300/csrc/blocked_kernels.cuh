@@ -57,6 +57,7 @@
 namespace gpr {
 
 constexpr int kBkThreads = 1024;
+constexpr int kRowBatch = 4;         // rows a thread finishes at a time
 constexpr int kMaxUnitSegs = 1024;  // segments of one expand unit (one per thread in the prefix scan)
 constexpr int kChunk = 256;         // edges per warp step: two runs of 4 consecutive edges per lane
 constexpr int kMaxUnitChunks = (1 << 20) / kChunk + kMaxUnitSegs;  // chunks of one expand unit
@@ -154,7 +155,8 @@ __device__ __forceinline__ void cp_async_wait() {
 __host__ __device__ constexpr size_t expand_ids_offset(int sb_bits) {
   return (((size_t)4 << sb_bits) + (size_t)(3 * kMaxUnitSegs + 1) * 4 + (size_t)kMaxUnitChunks * 2 + 15) & ~(size_t)15;
 }
-constexpr size_t kExpandStageBytes = (size_t)(kBkThreads / 32) * 128 * 8;
+constexpr int kExpandSlots = 4;  // chunks of source ids on their way per warp (a power of two)
+constexpr size_t kExpandStageBytes = (size_t)(kBkThreads / 32) * kExpandSlots * 64 * 8;
 // Shared memory of the accumulate kernel: two 32-bit words per row of the
 // bin, then per-warp staging slots (2 x (256 codes + 256 row ids)).
 constexpr size_t kAccumSlotBytes = kChunk * 4 + kChunk * 2;
@@ -177,11 +179,11 @@ __global__ void __launch_bounds__(kBkThreads, 1) bk_expand_kernel(
   int32_t* s_lo = s_pref + kMaxUnitSegs + 1;
   int32_t* s_hi = s_lo + kMaxUnitSegs;
   uint16_t* s_map = reinterpret_cast<uint16_t*>(s_hi + kMaxUnitSegs);  // chunk -> segment, kMaxUnitChunks
-  uint2* s_ids = reinterpret_cast<uint2*>(smem + expand_ids_offset(sb_bits));  // per warp: 2 slots x 64 x 8 bytes
+  uint2* s_ids = reinterpret_cast<uint2*>(smem + expand_ids_offset(sb_bits));  // per warp: kExpandSlots x 64 x 8 bytes
   __shared__ int32_t s_unit;
   __shared__ int32_t s_wsum[32];
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, nwarps = blockDim.x >> 5;
-  uint2* w_ids = s_ids + warp * 128;
+  uint2* w_ids = s_ids + warp * kExpandSlots * 64;
   for (;;) {
     __syncthreads();  // the previous unit is done with s_code and the segment tables
     if (tid == 0) s_unit = (int32_t)(atomicAdd(ctr, 1u) - epoch);
@@ -255,32 +257,30 @@ __global__ void __launch_bounds__(kBkThreads, 1) bk_expand_kernel(
     __syncthreads();
     // a warp takes chunks warp, warp + nwarps, ...; lane l handles edges
     // 4l..4l+3 and 128+4l..128+4l+3 of a chunk, whose 16-bit source ids it
-    // copies into its slot while the previous chunk is expanded
-    int32_t base = 0, lo = 0, hi = 0;
+    // copies into a slot while the chunks before it are expanded
     auto locate = [&](int32_t c, int32_t& b, int32_t& l, int32_t& h) {
       const int k = s_map[c];
       l = s_lo[k];
       h = s_hi[k];
       b = (l / kChunk + (c - s_pref[k])) * kChunk;
     };
-    auto stage = [&](int slot, int32_t b) {
-      cp_async8(w_ids + slot * 64 + lane, src_lo + b + 4 * lane);
-      cp_async8(w_ids + slot * 64 + 32 + lane, src_lo + b + 128 + 4 * lane);
-    };
-    if (warp < total) {
-      locate(warp, base, lo, hi);
-      stage(0, base);
-    }
-    cp_async_commit();
-    int slot = 0;
-    for (int32_t ch = warp; ch < total; ch += nwarps, slot ^= 1) {
-      int32_t nbase = 0, nlo = 0, nhi = 0;
-      if (ch + nwarps < total) {
-        locate(ch + nwarps, nbase, nlo, nhi);
-        stage(slot ^ 1, nbase);
+    auto stage = [&](int slot, int32_t c) {
+      if (c < total) {
+        int32_t b, l, h;
+        locate(c, b, l, h);
+        cp_async8(w_ids + slot * 64 + lane, src_lo + b + 4 * lane);
+        cp_async8(w_ids + slot * 64 + 32 + lane, src_lo + b + 128 + 4 * lane);
       }
       cp_async_commit();
-      cp_async_wait<1>();  // this lane's copies for the current chunk are in
+    };
+#pragma unroll
+    for (int k = 0; k < kExpandSlots - 1; ++k) stage(k, warp + k * nwarps);
+    int slot = 0;
+    for (int32_t ch = warp; ch < total; ch += nwarps, slot = (slot + 1) & (kExpandSlots - 1)) {
+      stage((slot + kExpandSlots - 1) & (kExpandSlots - 1), ch + (kExpandSlots - 1) * nwarps);
+      cp_async_wait<kExpandSlots - 1>();  // this lane's copies for the current chunk are in
+      int32_t base, lo, hi;
+      locate(ch, base, lo, hi);
 #pragma unroll
       for (int h = 0; h < 2; ++h) {
         const uint2 q = w_ids[slot * 64 + h * 32 + lane];
@@ -294,9 +294,6 @@ __global__ void __launch_bounds__(kBkThreads, 1) bk_expand_kernel(
             if (g + j >= lo && g + j < hi) vals[g + j] = s_code[id[j]];
         }
       }
-      base = nbase;
-      lo = nlo;
-      hi = nhi;
     }
     cp_async_wait<0>();
   }
@@ -334,6 +331,31 @@ __device__ __forceinline__ void acc_add8(uint32_t a_lo, uint32_t hw, const uint3
   }
 }
 
+// The same for eight codes, whatever they are: codes below 2^31 in the whole
+// warp (nearly always) are the values, added in 32 bits; a carry is a low word
+// that wrapped around.
+__device__ __forceinline__ void acc_add8_codes(uint32_t a_lo, uint32_t hw, const uint32_t (&d)[8],
+                                               const uint32_t (&w)[8], int U) {
+  const uint32_t any = (w[0] | w[1] | w[2] | w[3]) | (w[4] | w[5] | w[6] | w[7]);
+  if (__any_sync(0xffffffffu, any >> 31)) {
+    unsigned long long q[8];
+#pragma unroll
+    for (int j = 0; j < 8; ++j) q[j] = value_of(w[j], U);
+    acc_add8(a_lo, hw, d, q);
+    return;
+  }
+  uint32_t old[8];
+#pragma unroll
+  for (int j = 0; j < 8; ++j) old[j] = atom_add(a_lo + 4u * d[j], w[j]);
+  uint32_t up = 0;
+#pragma unroll
+  for (int j = 0; j < 8; ++j) up |= (uint32_t)(old[j] + w[j] < w[j]) << j;
+  if (__any_sync(0xffffffffu, up != 0u)) {
+#pragma unroll
+    for (int j = 0; j < 8; ++j) red_add_nonzero(a_lo + hw + 4u * d[j], (up >> j) & 1u);
+  }
+}
+
 // Edge index of slot j of this lane in a 256-edge chunk at `base`: lane l
 // holds edges 4l..4l+3 and 128+4l..128+4l+3.
 __device__ __forceinline__ int32_t chunk_edge(int32_t base, int lane, int j) {
@@ -349,7 +371,8 @@ __global__ void __launch_bounds__(kBkThreads, 1) bk_accum_kernel(
     float* __restrict__ x_out, uint32_t* __restrict__ c_out, StepParams* __restrict__ prm,
     double* __restrict__ partials, int32_t nbins, double* __restrict__ log_row) {
   extern __shared__ __align__(16) uint32_t s_acc32[];
-  __shared__ int32_t s_unit;
+  __shared__ int32_t s_unit[2];
+  __shared__ AccumUnit s_un[2];
   __shared__ int s_flag;
   const int32_t W = 1 << w_bits;
   uint32_t* s_lo = s_acc32;      // low words of the row accumulators
@@ -359,17 +382,28 @@ __global__ void __launch_bounds__(kBkThreads, 1) bk_accum_kernel(
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, nwarps = blockDim.x >> 5;
   // this warp's two staging slots: 256 codes or packed words, then 256 row ids
   unsigned char* w_stage = reinterpret_cast<unsigned char*>(s_acc32 + 2 * W) + (size_t)warp * 2 * kAccumSlotBytes;
-  for (;;) {
+  // thread 0 fetches the next unit while the current one is added
+  auto fetch = [&](int at) {
+    const int32_t u = (int32_t)(atomicAdd(ctr + 1, 1u) - epoch);
+    const bool ok = u >= 0 && u < nunits;
+    if (ok) s_un[at] = units[u];
+    s_unit[at] = ok;
+  };
+  if (tid == 0) fetch(0);
+  for (int at = 0;; at ^= 1) {
     __syncthreads();
-    if (tid == 0) s_unit = (int32_t)(atomicAdd(ctr + 1, 1u) - epoch);
-    __syncthreads();
-    const int32_t u = s_unit;
-    if (u < 0 || u >= nunits) return;
-    const AccumUnit un = units[u];
+    if (!s_unit[at]) return;
+    const AccumUnit un = s_un[at];
     const int32_t v0 = un.b << w_bits;
     const int32_t nv = min(W, n - v0);
-    for (int32_t i = tid; i < nv; i += blockDim.x) s_lo[i] = s_hi[i] = 0u;
+    {
+      const int32_t nq = (nv + 3) / 4;  // (W is a multiple of 4)
+      uint4* z_lo = reinterpret_cast<uint4*>(s_lo);
+      uint4* z_hi = reinterpret_cast<uint4*>(s_hi);
+      for (int32_t i = tid; i < nq; i += blockDim.x) z_lo[i] = z_hi[i] = make_uint4(0u, 0u, 0u, 0u);
+    }
     __syncthreads();
+    if (tid == 0) fetch(at ^ 1);
     // Lane l handles edges 4l..4l+3 and 128+4l..128+4l+3 of each 256-edge
     // chunk; it copies exactly those words (and row ids) into its slot while
     // the previous chunk is added.  An edge outside the unit's range (in a
@@ -377,50 +411,49 @@ __global__ void __launch_bounds__(kBkThreads, 1) bk_accum_kernel(
     //
     // Dense sources, edges [lo, mid): each word packs the source and the row;
     // the source's code is read from c_in (at most 1 MB of codes, kept in
-    // cache: a chunk's edges come from few, consecutive sources).
-    {
-      auto stage = [&](int slot, int32_t b) {
-        unsigned char* st = w_stage + slot * kAccumSlotBytes;
-        cp_async16(st + 16 * lane, vals + b + 4 * lane);
-        cp_async16(st + 512 + 16 * lane, vals + b + 128 + 4 * lane);
-      };
-      const int32_t first = (un.lo & ~(kChunk - 1)) + warp * kChunk;
-      if (first < un.mid) stage(0, first);
-      cp_async_commit();
-      int slot = 0;
-      for (int32_t base = first; base < un.mid; base += nwarps * kChunk, slot ^= 1) {
-        if (base + nwarps * kChunk < un.mid) stage(slot ^ 1, base + nwarps * kChunk);
+    // cache: a chunk's edges come from few, consecutive sources).  Words are
+    // copied two chunks ahead.  (Codes a chunk ahead as well, in 768 threads'
+    // registers, measured the same: 32 warps hide them as well.)  (Starting each unit at
+    // another place of its edges, so that the SMs are not at the same sources at
+    // one time, measured the same too.)
+    if (un.mid > un.lo) {
+      const int32_t c0 = un.lo / kChunk, nch = (un.mid - 1) / kChunk - c0 + 1;
+      auto chunk_at = [&](int32_t k) { return (c0 + k) * kChunk; };
+      auto stage = [&](int slot, int32_t k) {
+        if (k < nch) {
+          const int32_t b = chunk_at(k);
+          unsigned char* st = w_stage + slot * kAccumSlotBytes;
+          cp_async16(st + 16 * lane, vals + b + 4 * lane);
+          cp_async16(st + 512 + 16 * lane, vals + b + 128 + 4 * lane);
+        }
         cp_async_commit();
+      };
+      stage(0, warp);
+      stage(1, warp + nwarps);
+      for (int32_t k = warp, slot = 0; k < nch; k += nwarps, slot ^= 1) {
         cp_async_wait<1>();
         const unsigned char* st = w_stage + slot * kAccumSlotBytes;
         const uint4 wa = *reinterpret_cast<const uint4*>(st + 16 * lane);
         const uint4 wb = *reinterpret_cast<const uint4*>(st + 512 + 16 * lane);
-        uint32_t w[8] = {wa.x, wa.y, wa.z, wa.w, wb.x, wb.y, wb.z, wb.w};
-        uint32_t offm = 0;  // edges outside the range: word 0 (source 0, row 0), value 0
-        if (base < un.lo || base + kChunk > un.mid) {
+        const uint32_t w[8] = {wa.x, wa.y, wa.z, wa.w, wb.x, wb.y, wb.z, wb.w};
+        const int32_t b = chunk_at(k);
+        uint32_t d[8], cw[8];
+        if (b >= un.lo && b + kChunk <= un.mid) {
+#pragma unroll
+          for (int j = 0; j < 8; ++j) cw[j] = __ldg(c_in + (w[j] & dmask));
+#pragma unroll
+          for (int j = 0; j < 8; ++j) d[j] = w[j] >> dense_bits;
+        } else {
 #pragma unroll
           for (int j = 0; j < 8; ++j) {
-            const int32_t e = chunk_edge(base, lane, j);
-            if (e < un.lo || e >= un.mid) {
-              w[j] = 0u;
-              offm |= 1u << j;
-            }
+            const int32_t e = chunk_edge(b, lane, j);
+            const bool in = e >= un.lo && e < un.mid;
+            cw[j] = in ? __ldg(c_in + (w[j] & dmask)) : 0u;  // adds 0 to row 0
+            d[j] = in ? w[j] >> dense_bits : 0u;
           }
         }
-        uint32_t cw[8];
-#pragma unroll
-        for (int j = 0; j < 8; ++j) cw[j] = __ldg(c_in + (w[j] & dmask));
-        unsigned long long q[8];
-        codes_to_values(cw, U, q);
-        if (offm) {
-#pragma unroll
-          for (int j = 0; j < 8; ++j)
-            if ((offm >> j) & 1u) q[j] = 0ull;
-        }
-        uint32_t d[8];
-#pragma unroll
-        for (int j = 0; j < 8; ++j) d[j] = w[j] >> dense_bits;
-        acc_add8(a_lo, hw, d, q);
+        stage(slot, k + 2 * nwarps);  // (the words above are in registers: the codes' addresses came from them)
+        acc_add8_codes(a_lo, hw, d, cw, U);
       }
       cp_async_wait<0>();
     }
@@ -459,6 +492,11 @@ __global__ void __launch_bounds__(kBkThreads, 1) bk_accum_kernel(
               d[j] = 0u;
             }
           }
+        }
+        // no run of four edges of one row: eight additions as they are
+        if (!__any_sync(0xffffffffu, d[0] == d[3] || d[4] == d[7])) {
+          acc_add8_codes(a_lo, hw, d, w, U);
+          continue;
         }
         unsigned long long q[8];
         codes_to_values(w, U, q);
@@ -505,11 +543,24 @@ __global__ void __launch_bounds__(kBkThreads, 1) bk_accum_kernel(
       __syncthreads();
       if (!s_flag) continue;
       __threadfence();
-      // the last unit of the bin takes the totals and clears them for the next step
-      for (int32_t i = tid; i < nv; i += blockDim.x) {
-        const unsigned long long a = atomicExch(g + i, 0ull);
-        s_lo[i] = (uint32_t)a;
-        s_hi[i] = (uint32_t)(a >> 32);
+      // the last unit of the bin takes the totals and clears them for the next
+      // step (every unit has arrived: plain loads, several in flight)
+      for (int32_t i0 = tid; i0 < nv; i0 += kRowBatch * blockDim.x) {
+        unsigned long long a[kRowBatch];
+#pragma unroll
+        for (int j = 0; j < kRowBatch; ++j) {
+          const int32_t i = i0 + j * blockDim.x;
+          a[j] = i < nv ? __ldcg(g + i) : 0ull;
+        }
+#pragma unroll
+        for (int j = 0; j < kRowBatch; ++j) {
+          const int32_t i = i0 + j * blockDim.x;
+          if (i < nv) {
+            s_lo[i] = (uint32_t)a[j];
+            s_hi[i] = (uint32_t)(a[j] >> 32);
+            g[i] = 0ull;
+          }
+        }
       }
       if (tid == 0) bin_arrive[un.split] = 0;
       __syncthreads();
@@ -517,16 +568,29 @@ __global__ void __launch_bounds__(kBkThreads, 1) bk_accum_kernel(
     // finish the bin's rows: x' = coefB + coefA y, c' = code(T(x' / outdeg))
     const float A = prm->coefA, Bc = prm->coefB;
     float mass = 0.f, dang = 0.f, res = 0.f;
-    for (int32_t i = tid; i < nv; i += blockDim.x) {
-      const float y = from_fixed(((unsigned long long)s_hi[i] << 32) | s_lo[i], U);
-      const int32_t r = v0 + i;
-      const float idg = inv_deg[r];
-      const float xs = fmaf(A, y, Bc);
-      x_out[r] = xs;
-      c_out[r] = code_of(round_store(xs * idg, (T*)nullptr), U);
-      mass += xs;
-      res += fabsf(xs - x_in[r]);
-      if (idg == 0.0f) dang += xs;
+    // (several rows' loads in flight: one at a time left their latency, 16
+    // times a bin, a tenth of the kernel)
+    for (int32_t i0 = tid; i0 < nv; i0 += kRowBatch * blockDim.x) {
+      float idg[kRowBatch], xo[kRowBatch];
+#pragma unroll
+      for (int j = 0; j < kRowBatch; ++j) {
+        const int32_t i = i0 + j * blockDim.x;
+        idg[j] = i < nv ? __ldg(inv_deg + v0 + i) : 0.f;
+        xo[j] = i < nv ? x_in[v0 + i] : 0.f;
+      }
+#pragma unroll
+      for (int j = 0; j < kRowBatch; ++j) {
+        const int32_t i = i0 + j * blockDim.x;
+        if (i >= nv) break;
+        const int32_t r = v0 + i;
+        const float y = from_fixed(((unsigned long long)s_hi[i] << 32) | s_lo[i], U);
+        const float xs = fmaf(A, y, Bc);
+        x_out[r] = xs;
+        c_out[r] = code_of(round_store(xs * idg[j], (T*)nullptr), U);
+        mass += xs;
+        res += fabsf(xs - xo[j]);
+        if (idg[j] == 0.0f) dang += xs;
+      }
     }
     block_partials3(mass, dang, res, partials + 3 * (int64_t)un.b);
     if (tid == 0) {
