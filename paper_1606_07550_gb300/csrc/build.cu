@@ -176,16 +176,17 @@ SortScratch::~SortScratch() {
 }
 
 // ------------------------------------------------------------ histograms --
-// Digits of an LSD sort of `bits`-bit keys: 8-bit digits, or, where that takes
-// a pass fewer, the last (bits - 8 * passes) digits 9 bits wide; with 9-bit
-// digits the passes cover exactly `bits` bits, with 8-bit ones whole bytes.
-DigitPlan digit_plan(int bits) {
+// Digits of an LSD sort on bits [low, bits): 8-bit digits, or, where that takes
+// a pass fewer, the last of them 9 bits wide; with 9-bit digits the passes
+// cover exactly those bits, with 8-bit ones whole bytes from `low` on.
+DigitPlan digit_plan(int bits, int low) {
   DigitPlan d{};
-  bits = std::max(0, std::min(bits, 64));
+  low = std::max(0, low);
+  bits = std::max(0, std::min(bits, 64) - low);
   const int p8 = (bits + 7) / 8, p9 = (bits + 8) / 9;
   d.passes = p9 < p8 ? p9 : p8;
   const int nine = p9 < p8 ? bits - 8 * p9 : 0;  // the last `nine` passes are 9 bits wide
-  int sh = 0;
+  int sh = low;
   for (int p = 0; p < d.passes; ++p) {
     d.shift[p] = sh;
     d.width[p] = p >= d.passes - nine ? 9 : 8;
@@ -239,7 +240,9 @@ __global__ void digit_starts_kernel(const uint32_t* __restrict__ hist, DigitPlan
 // (warp, item, lane) order is input order and the per-warp match-based
 // ranking keeps the sort stable.  Thread t owns digits kDPT*t .. kDPT*t +
 // kDPT - 1 for the tile's scans and look-backs.
-template <int kBits, int kShift>
+// kBatch: predecessors read per look-back round trip; a sort of few tiles, all
+// resident at once and each waiting on the others' counts, takes more.
+template <int kBits, int kShift, int kBatch = 4>
 __global__ void __launch_bounds__(kThreads, 4) onesweep_kernel(
     const uint64_t* __restrict__ in, uint64_t* __restrict__ out, int64_t n, int shift_arg,
     const uint32_t* __restrict__ dstart, uint64_t* __restrict__ status, uint32_t* __restrict__ tile_ctr,
@@ -344,7 +347,7 @@ __global__ void __launch_bounds__(kThreads, 4) onesweep_kernel(
     const int d = kDPT * t + q;
     uint64_t excl = 0;
     if (tile != 0) {
-      excl = lookback(status + d, tile, kRadix, epoch, derr);
+      excl = lookback<kBatch>(status + d, tile, kRadix, epoch, derr);
       st_relaxed_u64(status + tile * kRadix + d, lb_word(epoch, kFlagInc, excl + cnt[q]));
     }
     // output index of tile position i with digit d: s_goff[d] + i (the digit's
@@ -373,11 +376,16 @@ using SweepKernel = void (*)(const uint64_t*, uint64_t*, int64_t, int, const uin
 static const SweepKernel kSweep8[8] = {onesweep_kernel<8, 0>,  onesweep_kernel<8, 8>,  onesweep_kernel<8, 16>,
                                        onesweep_kernel<8, 24>, onesweep_kernel<8, 32>, onesweep_kernel<8, 40>,
                                        onesweep_kernel<8, 48>, onesweep_kernel<8, 56>};
+static const SweepKernel kSweep8Any = onesweep_kernel<8, -1>;
 static const SweepKernel kSweep9 = onesweep_kernel<9, -1>;
+// sorts of up to kFewTiles tiles
+static const SweepKernel kSweep8Few = onesweep_kernel<8, -1, 16>;
+static const SweepKernel kSweep9Few = onesweep_kernel<9, -1, 16>;
+constexpr int64_t kFewTiles = 152;
 
 uint64_t* radix_sort_u64(uint64_t* keys, uint64_t* alt, int64_t n, int bits, cudaStream_t s,
-                         int* derr, uint32_t* hist_in) {
-  const DigitPlan dp = digit_plan(bits);
+                         int* derr, uint32_t* hist_in, int low) {
+  const DigitPlan dp = digit_plan(bits, low);
   const int passes = dp.passes;
   if (n <= 1 || passes == 0) return keys;
   const int64_t tiles = (n + kTile - 1) / kTile;
@@ -410,14 +418,18 @@ uint64_t* radix_sort_u64(uint64_t* keys, uint64_t* alt, int64_t n, int bits, cud
     std::call_once(carveout, [] {
       for (SweepKernel f : kSweep8)
         cudaFuncSetAttribute(f, cudaFuncAttributePreferredSharedMemoryCarveout, (int)cudaSharedmemCarveoutMaxShared);
-      cudaFuncSetAttribute(kSweep9, cudaFuncAttributePreferredSharedMemoryCarveout,
-                           (int)cudaSharedmemCarveoutMaxShared);
+      for (SweepKernel f : {kSweep8Any, kSweep9, kSweep8Few, kSweep9Few})
+        cudaFuncSetAttribute(f, cudaFuncAttributePreferredSharedMemoryCarveout, (int)cudaSharedmemCarveoutMaxShared);
     });
     uint64_t* a = keys;
     uint64_t* b = alt;
     for (int p = 0; p < passes; ++p) {
-      // 8-bit digits start at whole bytes until the first 9-bit one
-      const SweepKernel f = dp.width[p] == 9 ? kSweep9 : kSweep8[dp.shift[p] / 8];
+      // (8-bit digits of a whole sort start at whole bytes until the first 9-bit one)
+      const bool few = tiles <= kFewTiles;
+      const SweepKernel f = dp.width[p] == 9          ? (few ? kSweep9Few : kSweep9)
+                            : few                     ? kSweep8Few
+                            : (dp.shift[p] % 8) == 0 ? kSweep8[dp.shift[p] / 8]
+                                                      : kSweep8Any;
       f<<<(unsigned)tiles, kThreads, 0, s>>>(a, b, n, dp.shift[p], starts + kMaxRadix * p, status, ctr + p,
                                              (uint32_t)(p + 1), derr);
       GPR_CUDA(cudaGetLastError());
@@ -728,14 +740,16 @@ static int resident_grid(K kernel) {
 // Sorted unique-or-not keys (length m_keys) -> CSC arrays; returns m.
 // degree_from_raw: outdeg already holds each source's count of non-loop keys
 // (duplicates included), and the de-duplication subtracts the duplicates;
-// otherwise outdeg is counted from the kept keys.
+// otherwise outdeg is counted from the kept keys.  low: the keys ascend on
+// their low `low` bits already.  herr: where the error bits go, read back with m.
 static int64_t keys_to_csc(uint64_t* keys, uint64_t* alt, int64_t m_keys, int b, int32_t n, uint32_t* hist,
                            int32_t* col_ptr, int32_t* row_idx, int32_t* outdeg, int* derr, Temps& tmp,
-                           cudaStream_t s, bool presorted = false, bool degree_from_raw = false) {
+                           cudaStream_t s, bool presorted = false, bool degree_from_raw = false, int low = 0,
+                           int* herr = nullptr) {
   GPR_CUDA(cudaMemsetAsync(col_ptr, 0, ((size_t)n + 1) * 4, s));
   if (!degree_from_raw) GPR_CUDA(cudaMemsetAsync(outdeg, 0, (size_t)n * 4, s));
   if (m_keys == 0) return 0;
-  uint64_t* sorted = presorted ? keys : radix_sort_u64(keys, alt, m_keys, 2 * b, s, derr, hist);
+  uint64_t* sorted = presorted ? keys : radix_sort_u64(keys, alt, m_keys, 2 * b, s, derr, hist, low);
   trace_phase("build: sort", s);
   const int64_t tiles = (m_keys + kTile - 1) / kTile;
   uint64_t* status = (uint64_t*)tmp.get((size_t)tiles * 8);
@@ -759,6 +773,7 @@ static int64_t keys_to_csc(uint64_t* keys, uint64_t* alt, int64_t m_keys, int b,
   count_launches(1);
   int64_t m = 0;
   GPR_CUDA(cudaMemcpyAsync(&m, m_dev, sizeof m, cudaMemcpyDeviceToHost, s));
+  if (herr) GPR_CUDA(cudaMemcpyAsync(herr, derr, 4, cudaMemcpyDeviceToHost, s));
   GPR_CUDA(cudaStreamSynchronize(s));
   return m;
 }
@@ -774,7 +789,7 @@ __global__ void __launch_bounds__(kThreads) transpose_keys_kernel(const int32_t*
 }
 
 void graph_free_device(gpr_graph* g, cudaStream_t s);
-void plan_build(gpr_graph* g, cudaStream_t s, int* derr);
+void plan_build(gpr_graph* g, cudaStream_t s);
 
 // The copy stream and events of a chunked host-to-device COO copy, one set
 // per device, made on first use and kept for the process.  Builds that take
@@ -827,9 +842,8 @@ gpr_status build_graph(const int32_t* src_in, const int32_t* dst_in, int64_t m_r
     const int32_t* dst = dst_in;
     // 1. relabelling pi: nodes by descending raw out-degree (ties: ascending id)
     int32_t* odeg = (int32_t*)tmp.get((size_t)n * 4);
-    int32_t* maxd = (int32_t*)tmp.get(8);
+    int32_t* maxd = (int32_t*)derr + 1;  // beside the error bits: read back together
     GPR_CUDA(cudaMemsetAsync(odeg, 0, (size_t)n * 4, s));
-    GPR_CUDA(cudaMemsetAsync(maxd, 0, 8, s));
     if ((flags & GPR_PTR_HOST) && m_raw > 0) {
       // a host COO goes up in chunks on a copy stream; each chunk's raw
       // out-degrees are counted on `s` while the next chunk is in flight
@@ -863,11 +877,11 @@ gpr_status build_graph(const int32_t* src_in, const int32_t* dst_in, int64_t m_r
     max_kernel<<<grid_for(n), kThreads, 0, s>>>(odeg, n, maxd);
     GPR_CUDA(cudaGetLastError());
     count_launches(1);
-    int32_t hmax = 0;
-    int herr = 0;
-    GPR_CUDA(cudaMemcpyAsync(&hmax, maxd, 4, cudaMemcpyDeviceToHost, s));
-    GPR_CUDA(cudaMemcpyAsync(&herr, derr, 4, cudaMemcpyDeviceToHost, s));
+    int32_t back[2] = {0, 0};  // error bits, largest out-degree
+    GPR_CUDA(cudaMemcpyAsync(back, derr, sizeof back, cudaMemcpyDeviceToHost, s));
     GPR_CUDA(cudaStreamSynchronize(s));
+    int herr = back[0];
+    const int32_t hmax = back[1];
     if (herr & DERR_BAD_ID) throw StatusFail{GPR_EINVAL, "graph_build: an edge id is outside [0, n)"};
     trace_phase("build: raw out-degrees", s);
     {
@@ -876,7 +890,8 @@ gpr_status build_graph(const int32_t* src_in, const int32_t* dst_in, int64_t m_r
       node_order_keys_kernel<<<grid_for(n), kThreads, 0, s>>>(odeg, n, b, hmax, nk);
       GPR_CUDA(cudaGetLastError());
       count_launches(1);
-      uint64_t* ns = radix_sort_u64(nk, na, n, b + bits_for((uint32_t)hmax), s, derr, nullptr);
+      // (the keys ascend by id already: only the degrees are sorted)
+      uint64_t* ns = radix_sort_u64(nk, na, n, b + bits_for((uint32_t)hmax), s, derr, nullptr, b);
       g->plan.new2old = (int32_t*)dalloc((size_t)n * 4, s);
       g->plan.old2new = (int32_t*)dalloc((size_t)n * 4, s);
       perm_from_sorted_kernel<<<grid_for(n), kThreads, 0, s>>>(ns, n, (1ull << b) - 1, g->plan.new2old,
@@ -911,9 +926,7 @@ gpr_status build_graph(const int32_t* src_in, const int32_t* dst_in, int64_t m_r
       count_launches(1);
       trace_phase("build: pack", s);
       m = keys_to_csc(keys, alt, m_raw, b, n, hist, g->col_ptr, row_idx_full, g->outdeg, derr, tmp, s,
-                      /*presorted=*/false, /*degree_from_raw=*/true);
-      GPR_CUDA(cudaMemcpyAsync(&herr, derr, 4, cudaMemcpyDeviceToHost, s));
-      GPR_CUDA(cudaStreamSynchronize(s));
+                      /*presorted=*/false, /*degree_from_raw=*/true, /*low=*/0, &herr);
       if (herr & DERR_TIMEOUT) throw StatusFail{GPR_ETIMEOUT, "graph_build: a device-side wait timed out"};
     } else {
       GPR_CUDA(cudaMemsetAsync(g->col_ptr, 0, ((size_t)n + 1) * 4, s));
@@ -929,18 +942,8 @@ gpr_status build_graph(const int32_t* src_in, const int32_t* dst_in, int64_t m_r
     tmp.release();
     trace_phase("build: dedupe", s);
     // 3. execution layout (degree buckets, chunks, inverse degrees)
-    int* derr2 = (int*)dalloc(8, s);
-    GPR_CUDA(cudaMemsetAsync(derr2, 0, 8, s));
-    try {
-      plan_build(g, s, derr2);
-    } catch (...) {
-      dfree(derr2, s);
-      throw;
-    }
-    GPR_CUDA(cudaMemcpyAsync(&herr, derr2, 4, cudaMemcpyDeviceToHost, s));
+    plan_build(g, s);
     GPR_CUDA(cudaStreamSynchronize(s));
-    dfree(derr2, s);
-    if (herr & DERR_TIMEOUT) throw StatusFail{GPR_ETIMEOUT, "graph_build: a device-side wait timed out"};
     trace_phase("build: plan", s);
     *out = g;
     return GPR_OK;
@@ -988,13 +991,15 @@ gpr_graph* build_transposed(const gpr_graph* g, cudaStream_t s) {
                                                                                      b, keys);
       GPR_CUDA(cudaGetLastError());
       count_launches(1);
-      m = keys_to_csc(keys, alt, g->m, b, n, nullptr, t->col_ptr, t->row_idx, t->outdeg, derr, tmp, s);
+      // (the keys come in order of destination: only the sources are sorted)
+      m = keys_to_csc(keys, alt, g->m, b, n, nullptr, t->col_ptr, t->row_idx, t->outdeg, derr, tmp, s,
+                      /*presorted=*/false, /*degree_from_raw=*/false, /*low=*/b);
     } else {
       GPR_CUDA(cudaMemsetAsync(t->col_ptr, 0, ((size_t)n + 1) * 4, s));
       GPR_CUDA(cudaMemsetAsync(t->outdeg, 0, (size_t)n * 4, s));
     }
     t->m = m;
-    plan_build(t, s, derr);
+    plan_build(t, s);
     int herr = 0;
     GPR_CUDA(cudaMemcpyAsync(&herr, derr, 4, cudaMemcpyDeviceToHost, s));
     GPR_CUDA(cudaStreamSynchronize(s));
@@ -1359,18 +1364,8 @@ gpr_status update_graph(gpr_graph* g, const int32_t* ins_src, const int32_t* ins
     new_col_ptr = new_row_idx = new_outdeg = nullptr;
     g->m = m2;
     g->m_raw = m2;
-    int* derr2 = (int*)dalloc(8, s);
-    GPR_CUDA(cudaMemsetAsync(derr2, 0, 8, s));
-    try {
-      plan_build(g, s, derr2);
-    } catch (...) {
-      dfree(derr2, s);
-      throw;
-    }
-    GPR_CUDA(cudaMemcpyAsync(&herr, derr2, 4, cudaMemcpyDeviceToHost, s));
+    plan_build(g, s);
     GPR_CUDA(cudaStreamSynchronize(s));
-    dfree(derr2, s);
-    if (herr & DERR_TIMEOUT) throw StatusFail{GPR_ETIMEOUT, "graph_update: a device-side wait timed out"};
     return GPR_OK;
   } catch (const StatusFail& f) {
     tmp.release();
@@ -1400,6 +1395,7 @@ gpr_status export_graph(const gpr_graph* g, int32_t* col_ptr_h, int32_t* row_idx
     const int64_t m = g->m;
     const int b = g->id_bits;
     int* derr = (int*)tmp.get(8);
+    int herr = 0;
     GPR_CUDA(cudaMemsetAsync(derr, 0, 8, s));
     int32_t* cp = (int32_t*)tmp.get(((size_t)n + 1) * 4);
     int32_t* ri = (int32_t*)tmp.get((size_t)std::max<int64_t>(m, 1) * 4);
@@ -1410,7 +1406,7 @@ gpr_status export_graph(const gpr_graph* g, int32_t* col_ptr_h, int32_t* row_idx
       csc_keys_kernel<<<grid_for(m), kThreads, 0, s>>>(g->col_ptr, g->row_idx, n, m, b, g->plan.new2old, keys);
       GPR_CUDA(cudaGetLastError());
       count_launches(1);
-      const int64_t m2 = keys_to_csc(keys, alt, m, b, n, nullptr, cp, ri, od, derr, tmp, s);
+      const int64_t m2 = keys_to_csc(keys, alt, m, b, n, nullptr, cp, ri, od, derr, tmp, s, false, false, 0, &herr);
       if (m2 != m) throw StatusFail{GPR_ECUDA, "graph_export: edge count changed under relabelling"};
     } else {
       GPR_CUDA(cudaMemsetAsync(cp, 0, ((size_t)n + 1) * 4, s));
@@ -1419,8 +1415,6 @@ gpr_status export_graph(const gpr_graph* g, int32_t* col_ptr_h, int32_t* row_idx
     if (col_ptr_h) GPR_CUDA(cudaMemcpy(col_ptr_h, cp, ((size_t)n + 1) * 4, cudaMemcpyDeviceToHost));
     if (row_idx_h && m > 0) GPR_CUDA(cudaMemcpy(row_idx_h, ri, (size_t)m * 4, cudaMemcpyDeviceToHost));
     if (outdeg_h) GPR_CUDA(cudaMemcpy(outdeg_h, od, (size_t)n * 4, cudaMemcpyDeviceToHost));
-    int herr = 0;
-    GPR_CUDA(cudaMemcpy(&herr, derr, 4, cudaMemcpyDeviceToHost));
     tmp.release();
     GPR_CUDA(cudaStreamSynchronize(s));
     if (herr & DERR_TIMEOUT) throw StatusFail{GPR_ETIMEOUT, "graph_export: a device-side wait timed out"};

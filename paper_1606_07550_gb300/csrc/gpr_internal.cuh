@@ -97,15 +97,16 @@ struct DigitPlan {
   int shift[kMaxPasses];
   int width[kMaxPasses];
 };
-DigitPlan digit_plan(int bits);
+DigitPlan digit_plan(int bits, int low = 0);
 
-// Sorts keys[0..n) ascending on the low `bits` bits (stable LSD, the digits of
-// digit_plan(bits)), using `alt` (n entries) as the second buffer.  Returns
+// Sorts keys[0..n) ascending on bits [low, bits) (stable LSD, the digits of
+// digit_plan(bits, low)), using `alt` (n entries) as the second buffer: keys
+// that already ascend on their low bits end ascending on all `bits`.  Returns
 // the buffer holding the result (keys or alt).  hist: the caller already
-// filled it (passes x kMaxRadix digit counts, device, digit_plan(bits)'s
-// digits); if null it is computed.
+// filled it (passes x kMaxRadix digit counts, device, the plan's digits); if
+// null it is computed.
 uint64_t* radix_sort_u64(uint64_t* keys, uint64_t* alt, int64_t n, int bits, cudaStream_t s,
-                         int* derr, uint32_t* hist = nullptr);
+                         int* derr, uint32_t* hist = nullptr, int low = 0);
 
 // ---- PageRank execution layout -------------------------------------------
 // The CSC is stored in relabelled ids (descending out-degree).  Rows are run
@@ -184,7 +185,7 @@ struct gpr_graph {
 };
 
 namespace gpr {
-void plan_build(gpr_graph* g, cudaStream_t s, int* derr);
+void plan_build(gpr_graph* g, cudaStream_t s);
 // The transposed graph of g (throws StatusFail / CudaFail).
 gpr_graph* build_transposed(const gpr_graph* g, cudaStream_t s);
 // The caller-id out-adjacency of g into two new device arrays (throws).
@@ -285,7 +286,7 @@ __device__ __forceinline__ uint64_t lb_word(uint32_t epoch, uint64_t flag, uint6
 // The words of kLookBatch predecessors are read at once, so one round trip to
 // L2 walks past up to kLookBatch aggregates.  Every wait is bounded; on
 // timeout it sets DERR_TIMEOUT and returns what it has.
-constexpr int kLookBatch = 4;
+template <int kLookBatch = 4>
 __device__ __forceinline__ uint64_t lookback(const uint64_t* status, int64_t tile, int64_t stride,
                                              uint32_t epoch, int* derr) {
   uint64_t excl = 0;

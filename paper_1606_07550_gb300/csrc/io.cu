@@ -187,13 +187,10 @@ gpr_status load_graph(const char* path, cudaStream_t s, gpr_graph** out) {
     GPR_CUDA(cudaStreamSynchronize(s));
     if (herr & IOERR_ROWS) throw StatusFail{GPR_EINVAL, "graph_load: a row's sources are out of range or unsorted"};
     if (herr & IOERR_PERM) throw StatusFail{GPR_EINVAL, "graph_load: new2old is not a permutation"};
-    GPR_CUDA(cudaMemsetAsync(err, 0, 8, s));
-    plan_build(g, s, err);
-    GPR_CUDA(cudaMemcpyAsync(&herr, err, 4, cudaMemcpyDeviceToHost, s));
+    plan_build(g, s);
     GPR_CUDA(cudaStreamSynchronize(s));
     dfree(err, s);
     err = nullptr;
-    if (herr & DERR_TIMEOUT) throw StatusFail{GPR_ETIMEOUT, "graph_load: a device-side wait timed out"};
     *out = g;
     return GPR_OK;
   } catch (const StatusFail& f) {

@@ -892,7 +892,9 @@ static void persist_layout(gpr_graph* g, PagerankWork* w, cudaStream_t s) {
     GPR_CUDA(cudaGetLastError());
     int32_t h[kPersShort + 2];
     GPR_CUDA(cudaMemcpyAsync(h, count, sizeof h, cudaMemcpyDeviceToHost, s));
-    const uint64_t* sorted = radix_sort_u64(keys, alt, n, b + ceil_log2((int64_t)g->max_in + 1), s, derr);
+    // (the keys ascend by row already: only the degrees are sorted)
+    const uint64_t* sorted =
+        radix_sort_u64(keys, alt, n, b + ceil_log2((int64_t)g->max_in + 1), s, derr, nullptr, b);
     GPR_CUDA(cudaStreamSynchronize(s));
     // slice widths: the in-degree of a slice's first row
     w->pers_long = h[kPersShort + 1];

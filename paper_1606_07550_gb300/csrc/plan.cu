@@ -79,6 +79,7 @@ struct Thresholds {
 };
 
 struct PlanDev {
+  int32_t derr;  // error bits of the sort
   int32_t n_dangling, max_in, max_out;
   int32_t bstart[kMaxBuckets + 1];
 };
@@ -213,7 +214,7 @@ static int grid_for(int64_t items) {
   return (int)std::max<int64_t>(1, std::min<int64_t>((items + kPThreads - 1) / kPThreads, (int64_t)num_sms() * 8));
 }
 
-void plan_build(gpr_graph* g, cudaStream_t s, int* derr) {
+void plan_build(gpr_graph* g, cudaStream_t s) {
   Plan& P = g->plan;
   const int32_t n = g->n;
   const int b = g->id_bits;
@@ -242,7 +243,8 @@ void plan_build(gpr_graph* g, cudaStream_t s, int* derr) {
     count_launches(1);
     int bb = 1;
     while ((1 << bb) < nb) ++bb;
-    uint64_t* sorted = radix_sort_u64(keys, alt, n, b + bb, s, derr, nullptr);
+    // (the keys ascend by row already: only the bucket is sorted)
+    uint64_t* sorted = radix_sort_u64(keys, alt, n, b + bb, s, &pd->derr, nullptr, b);
     trace_phase("plan: bucket keys + sort", s);
     row_lists_kernel<<<grid_for(n), kPThreads, 0, s>>>(sorted, n, b, P.rows, pd);
     GPR_CUDA(cudaGetLastError());
@@ -250,6 +252,7 @@ void plan_build(gpr_graph* g, cudaStream_t s, int* derr) {
     PlanDev h{};
     GPR_CUDA(cudaMemcpyAsync(&h, pd, sizeof h, cudaMemcpyDeviceToHost, s));
     GPR_CUDA(cudaStreamSynchronize(s));
+    if (h.derr & DERR_TIMEOUT) throw StatusFail{GPR_ETIMEOUT, "graph plan: a look-back wait of the sort timed out"};
     g->n_dangling = h.n_dangling;
     g->max_in = h.max_in;
     g->max_out = h.max_out;
