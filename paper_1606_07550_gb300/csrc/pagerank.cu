@@ -972,21 +972,24 @@ static void launch_persist(const PersistArgs& A, int blocks, size_t smem, cudaSt
   count_launches(1);
 }
 
-template <typename T>
-static void run_persist(gpr_graph* g, PagerankWork* w, double damping, int32_t iters, float* dst, cudaStream_t s) {
-  const Plan& P = g->plan;
-  const int32_t n = g->n;
-  const size_t need = 48 + ((size_t)iters + 1) * 24;
-  if (w->ctl_cap < need) {
-    dfree(w->ctl, s);
-    w->ctl = nullptr;
-    w->ctl_cap = 0;
-    const size_t cap = std::max<size_t>(need, 4096);
-    w->ctl = (char*)dalloc(cap, s);
-    w->ctl_cap = cap;
-  }
-  GPR_CUDA(cudaMemsetAsync(w->ctl, 0, need, s));
+// One product of the centralities (PersistArgs::product): no barrier, so an
+// ordinary launch.
+static void launch_product(const PersistArgs& A, int blocks, size_t smem, cudaStream_t s) {
+  GPR_CUDA(cudaFuncSetAttribute(persist_kernel<float, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+  persist_kernel<float, false><<<blocks, kPersThreads, smem, s>>>(A);
+  GPR_CUDA(cudaGetLastError());
+  count_launches(1);
+}
+
+static void split_pair(double v, float* hi, float* lo) {
+  *hi = (float)v;
+  *lo = (float)(v - (double)*hi);
+}
+
+// The layout's part of the arguments, for contributions of `size` bytes.
+static PersistArgs persist_args(const gpr_graph* g, const PagerankWork* w, double damping, int size) {
   PersistArgs A{};
+  const int32_t n = g->n;
   A.row_idx = g->row_idx;
   A.row = w->pers_row;
   A.inv = w->pers_inv;
@@ -996,11 +999,33 @@ static void run_persist(gpr_graph* g, PagerankWork* w, double damping, int32_t i
   A.deal = w->pers_deal;
   A.n_long = w->pers_long;
   A.nslices = w->pers_slices;
-  A.inv_deg = P.inv_deg;
-  A.old2new = P.old2new;
+  A.inv_deg = g->plan.inv_deg;
+  A.old2new = g->plan.old2new;
   A.n = n;
-  A.H = std::min<int32_t>(n, kPersHotBytes / (int)sizeof(T)) & ~7;
+  A.H = std::min<int32_t>(n, kPersHotBytes / size) & ~7;
   A.xi = w->pers_x;
+  split_pair(damping, &A.d_hi, &A.d_lo);
+  split_pair((1.0 - damping) / (double)n, &A.t_hi, &A.t_lo);
+  split_pair(1.0 / (double)n, &A.in_hi, &A.in_lo);
+  return A;
+}
+
+static void persist_ctl(PagerankWork* w, size_t need, cudaStream_t s) {
+  if (w->ctl_cap < need) {
+    dfree(w->ctl, s);
+    w->ctl = nullptr;
+    w->ctl_cap = 0;
+    const size_t cap = std::max<size_t>(need, 4096);
+    w->ctl = (char*)dalloc(cap, s);
+    w->ctl_cap = cap;
+  }
+  GPR_CUDA(cudaMemsetAsync(w->ctl, 0, need, s));
+}
+
+template <typename T>
+static void run_persist(gpr_graph* g, PagerankWork* w, double damping, int32_t iters, float* dst, cudaStream_t s) {
+  persist_ctl(w, 48 + ((size_t)iters + 1) * 24, s);
+  PersistArgs A = persist_args(g, w, damping, (int)sizeof(T));
   A.x = w->x[0];
   A.c[0] = w->c[0];
   A.c[1] = w->c[1];
@@ -1008,13 +1033,6 @@ static void run_persist(gpr_graph* g, PagerankWork* w, double damping, int32_t i
   A.log_row = (double*)(w->ctl + 16);
   A.sums = (unsigned long long*)(w->ctl + 48);
   A.out = dst;
-  auto split = [](double v, float* hi, float* lo) {
-    *hi = (float)v;
-    *lo = (float)(v - (double)*hi);
-  };
-  split(damping, &A.d_hi, &A.d_lo);
-  split((1.0 - damping) / (double)n, &A.t_hi, &A.t_lo);
-  split(1.0 / (double)n, &A.in_hi, &A.in_lo);
   A.iters = iters;
   const size_t smem = std::max<size_t>((size_t)A.H * sizeof(T), 16);
   if (w->pers_cluster)
@@ -1305,15 +1323,39 @@ gpr_status run_centrality(gpr_graph* g, int kind, int32_t iters, float* out_x, f
         blocked_record_reset(wt->blk, s);
       }
     }
+    // small graphs: the products of the single-launch kernel, each a launch of
+    // its own (ones as inverse degrees: pers_inv is PageRank's)
+    const bool small = !blocked && persist_eligible(g, w, kSchedPull, false) &&
+                       (kind == 0 || persist_eligible(t, wt, kSchedPull, false));
+    if (small) {
+      if (!w->pers) persist_layout(g, w, s);
+      if (kind == 1 && !wt->pers) persist_layout(t, wt, s);
+      persist_ctl(w, 48 + ((size_t)2 * iters + 1) * 24, s);
+    }
+    int32_t products = 0;
     int32_t it_g = 0, it_t = 0;  // steps since the reset, per layout
     auto product = [&](gpr_graph* gg, PagerankWork* ww, const float* c_in, const float* x_in, float* x_out,
                        float* c_out, double* log_row) {
-      if (blocked)  // the contributions are held as codes
+      if (small) {
+        PersistArgs A = persist_args(gg, ww, 1.0, 4);
+        A.inv = w->ones;
+        A.x = x_out;
+        A.c[0] = const_cast<float*>(c_in);
+        A.c[1] = c_out;
+        A.sums = (unsigned long long*)(w->ctl + 48) + 3 * (int64_t)products++;
+        A.iters = 1;
+        A.product = 1;
+        launch_product(A, ww->pers_blocks, std::max<size_t>((size_t)A.H * 4, 16), s);
+      } else if (blocked)  // the contributions are held as codes
         blocked_record_step<float>(ww->blk, gg, (const uint32_t*)c_in, x_in, x_out, (uint32_t*)c_out, w->ones,
                                    w->prm, log_row, gg == g ? it_g++ : it_t++, s);
       else
         launch_pull_step(gg, ww, s, c_in, x_in, x_out, c_out, w->ones, w->prm, log_row);
     };
+    if (small) {  // the start vector's largest entry
+      const float start = 1.0f / (float)n;
+      GPR_CUDA(cudaMemcpyAsync(w->ctl + 48, &start, 4, cudaMemcpyHostToDevice, s));
+    }
     ensure_log(w, 2 * iters + 2, s);
     const StepParams hp{0.f, 0.f, 1.0, (double)n};  // d = 1: no teleport, coefA = 1 / mass
     GPR_CUDA(cudaMemcpyAsync(w->prm, &hp, sizeof hp, cudaMemcpyHostToDevice, s));

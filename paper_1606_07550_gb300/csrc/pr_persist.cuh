@@ -27,6 +27,9 @@
 // kernels, then exact integer sums of multiples of 2^-60 over warps and blocks,
 // so runs are bitwise identical.
 //
+// The centralities take the same kernel a step at a time (PersistArgs::product):
+// one launch a product instead of six.
+//
 // The barrier's wait is bounded: after kSpinLimit polls a block sets the error
 // flag, writes NaN ranks and returns, and so do the others.
 #pragma once
@@ -69,6 +72,13 @@ struct PersistArgs {
   // damping, (1 - d) / n and 1 / n, each the sum of two floats
   float d_hi, d_lo, t_hi, t_lo, in_hi, in_lo;
   int32_t iters;
+  // 1: one product of a power iteration, x = y / (largest entry of the vector
+  // before; 0 if that is 0), from contributions and a largest entry that the
+  // caller or the product before left (no start vector, so no barrier); x and
+  // contributions stored, no output.  sums rows hold the largest entry's bits:
+  // a product can scale the vector by anything, which fixed-point sums would
+  // not follow, and its largest entry is exact in any order.
+  int32_t product;
 };
 
 constexpr int kPersFix = 60;
@@ -200,6 +210,11 @@ __global__ void __launch_bounds__(kPersThreads, 1) persist_kernel(const __grid_c
       if (lane == 0 && t) atomicAdd(A.sums + 3 * (int64_t)it + warp, t);
     }
   };
+  auto add_max = [&](int32_t it, float mx) {
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, o));
+    if (lane == 0 && mx > 0.f) atomicMax((unsigned int*)(A.sums + 3 * (int64_t)it), __float_as_uint(mx));
+  };
   constexpr double unit = 1.0 / (double)(1ull << kPersFix);
 
   // the block's long rows and their chunks
@@ -237,7 +252,7 @@ __global__ void __launch_bounds__(kPersThreads, 1) persist_kernel(const __grid_c
 
   // x_0 = 1/n and its contributions
   const float x0 = 1.0f / (float)n;
-  {
+  if (!A.product) {
     T* c0 = (T*)A.c[0];
     float mass = 0.f, dang = 0.f;
     for (int32_t v = blockIdx.x * kPersThreads + tid; v < n; v += nblk * kPersThreads) {
@@ -249,6 +264,7 @@ __global__ void __launch_bounds__(kPersThreads, 1) persist_kernel(const __grid_c
     }
     add_sums(0, mass, dang, 0.f);
   }
+  if (A.product) __syncthreads();  // (add_sums has one)
   const int32_t nchunks = s_first[nl];
 
   // a slice: this lane's row, its width and its first indices
@@ -280,7 +296,7 @@ __global__ void __launch_bounds__(kPersThreads, 1) persist_kernel(const __grid_c
   const bool single = warp + kPersWarps >= nsl;  // the warp's one slice stays in its registers
   Slice cur = load_slice(warp);
   float cx = x0;
-  barrier();
+  if (!A.product) barrier();
 
   for (int32_t it = 0; it < A.iters && !failed; ++it) {
     const T* cin = (const T*)A.c[it & 1];
@@ -288,7 +304,11 @@ __global__ void __launch_bounds__(kPersThreads, 1) persist_kernel(const __grid_c
     const bool last = it + 1 == A.iters;
     // the step's coefficients (warp 0) beside the copy of the first H contributions
     if (warp == 0) {
-      if (lane == 0) {
+      if (lane == 0 && A.product) {
+        const float m = __uint_as_float(__ldcg((const unsigned int*)(A.sums + 3 * (int64_t)it)));
+        s_coef[0] = m > 0.f ? 1.0f / m : 0.f;
+        s_coef[1] = 0.f;
+      } else if (lane == 0) {
         // mass and dangling mass as sums of two floats (48 bits; the FP64 pipe
         // would take longer than the rest of the step), 1 / mass by a Newton
         // step on the FP32 reciprocal
@@ -321,11 +341,9 @@ __global__ void __launch_bounds__(kPersThreads, 1) persist_kernel(const __grid_c
     auto finish = [&](int32_t i, int32_t r, float inv, float xo, float y) {
       const float xs = fmaf(ca, y, cb);
       A.xi[i] = xs;
-      if (last)
-        A.x[r] = xs;
-      else
-        store_rank(cout, r, xs * inv);
-      mass += xs;
+      if (last) A.x[r] = xs;
+      if (!last || A.product) store_rank(cout, r, xs * inv);
+      mass = A.product ? fmaxf(mass, xs) : mass + xs;
       res += fabsf(xs - xo);
       if (inv == 0.0f) dang += xs;
       return xs;
@@ -412,6 +430,10 @@ __global__ void __launch_bounds__(kPersThreads, 1) persist_kernel(const __grid_c
         const int32_t i = __ldg(my_long + tid);
         finish(i, __ldg(A.row + i), __ldg(A.inv + i), it > 0 ? A.xi[i] : x0, y);
       }
+    }
+    if (A.product) {
+      add_max(it + 1, mass);
+      return;
     }
     add_sums(it + 1, mass, dang, res);
     barrier();
