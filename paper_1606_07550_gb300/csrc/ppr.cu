@@ -243,30 +243,6 @@ __device__ __forceinline__ int32_t lower_bound_i32(const int32_t* a, int32_t n, 
   return lo;
 }
 
-// Rows [r0, r1) split into kPprWarps contiguous ranges of about equal
-// (edges + rows): warp w takes [first, last).  Deterministic, and balanced so
-// that no warp holds the block at its per-step barriers.
-__device__ __forceinline__ void warp_rows(const int32_t* __restrict__ col_ptr, int32_t r0, int32_t r1, int w,
-                                          int32_t& first, int32_t& last) {
-  const int64_t k0 = (int64_t)col_ptr[r0] + r0, k1 = (int64_t)col_ptr[r1] + r1;
-  auto at = [&](int ww) -> int32_t {
-    if (ww <= 0) return r0;
-    if (ww >= kPprWarps) return r1;
-    const int64_t target = k0 + (k1 - k0) * ww / kPprWarps;
-    int32_t lo = r0, hi = r1;  // first p in [r0, r1] with col_ptr[p] + p >= target
-    while (lo < hi) {
-      const int32_t mid = lo + (hi - lo) / 2;
-      if ((int64_t)col_ptr[mid] + mid < target)
-        lo = mid + 1;
-      else
-        hi = mid;
-    }
-    return lo;
-  };
-  first = at(w);
-  last = at(w + 1);
-}
-
 template <typename T>
 __global__ void __launch_bounds__(kPprThreads, 1) ppr_kernel(PprJob* __restrict__ jobs,
                                                             const int32_t* __restrict__ order, int32_t njobs,
@@ -521,326 +497,7 @@ __global__ void __launch_bounds__(kPprThreads, 1) ppr_kernel(PprJob* __restrict_
   }
 }
 
-// ---- step-major kernel (the server) ------------------------------------------
-//
-// One launch = one step of every (slot, part) item.  Launch sequence of a
-// tick with T steps: kStepInit (fresh columns start at e_seed; state st[0]),
-// kStepRun with step = 1..T (fold the previous step's part sums in part
-// order, decide stops, then pull), kStepFinish (fold step T, write the
-// records).  Run step s reads st[(s-1)&1] and psum[(s-1)&1] and writes
-// st[s&1] and psum[s&1]; every part of a slot computes the same decisions and
-// only part 0 writes them.  A finished column is written out, by node id,
-// by every part for its own rows, at the launch that detects it.
-
-template <typename T>
-__global__ void __launch_bounds__(kPprThreads, 1) ppr_step_kernel(const SlotDesc* __restrict__ slots,
-                                                                 const StepItem* __restrict__ items, int32_t nitems,
-                                                                 int mode, int32_t step) {
-  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-  __shared__ float s_wpart[kPprWarps][3][kPprCols];
-  __shared__ int32_t s_seed[kPprCols], s_status[kPprCols], s_iters[kPprCols], s_newdone[kPprCols];
-  __shared__ float s_d[kPprCols];
-  __shared__ double s_D[kPprCols];
-  __shared__ float s_bprev[kPprCols];  // seed coefficient of each column's previous step
-  const int cur = step & 1, prev = cur ^ 1;
-  for (int32_t ii = blockIdx.x; ii < nitems; ii += gridDim.x) {
-    const StepItem item = items[ii];
-    const SlotDesc* S = slots + item.slot;
-    const int32_t r0 = S->part_rows[item.part], r1 = S->part_rows[item.part + 1];
-    const float* __restrict__ inv_deg = S->inv_deg;
-    constexpr bool kDelta = std::is_same<T, __nv_bfloat16>::value;
-    float* X = kDelta ? nullptr : S->X;
-    float4* YS = kDelta ? S->YS : nullptr;
-
-    // ---- column state for this launch
-    if (tid < kPprCols) {
-      const PprCol cr = S->rec[tid];
-      const int32_t seed_row = cr.status == kColEmpty ? -1 : S->old2new[cr.seed];
-      s_seed[tid] = seed_row;
-      s_d[tid] = cr.damping;
-      int32_t status, iters, stall;
-      double D, res, best;
-      float bprev;  // seed coefficient of the column's latest executed step (1 before its first)
-      int newdone = 0;
-      if (mode == kStepInit) {
-        status = cr.status;
-        iters = cr.iters;
-        D = cr.dangling;
-        res = cr.residual;
-        best = cr.best;
-        stall = cr.stall;
-        bprev = cr.bused;
-        if (status == kColFresh) {
-          bprev = 1.f;
-          status = kColRunning;
-          iters = 0;
-          res = 0.0;
-          best = INFINITY;
-          stall = 0;
-          D = inv_deg[seed_row] == 0.f ? 1.0 : 0.0;
-          if (iters >= cr.max_iters) {
-            status = kColDone;
-            newdone = 1;
-          }
-        }
-      } else {
-        const ColState cs = S->st[prev][tid];
-        status = cs.status;
-        iters = cs.iters;
-        D = cs.dangling;
-        res = cs.residual;
-        best = cs.best;
-        stall = cs.stall;
-        bprev = cs.bused;
-        const bool fold = mode == kStepFinish || step > 1;
-        if (fold && status == kColRunning) {
-          double dsum = 0.0, rsum = 0.0;
-          const double* ps = S->psum[prev];
-          for (int32_t q = 0; q < S->nparts; ++q) {
-            dsum += ps[(3 * q + 1) * kPprCols + tid];
-            rsum += ps[(3 * q + 2) * kPprCols + tid];
-          }
-          D = dsum;
-          res = rsum;
-          iters += 1;
-          const double d = cr.damping;
-          if (rsum < best) {
-            best = rsum;
-            stall = 0;
-          } else {
-            ++stall;
-          }
-          if ((cr.tol > 0.f && ((d / (1.0 - d)) * rsum <= (double)cr.tol || stall >= kStallSteps)) ||
-              iters >= cr.max_iters) {
-            status = kColDone;
-            newdone = 1;
-          }
-        }
-      }
-      s_status[tid] = status;
-      s_iters[tid] = iters;
-      s_D[tid] = D;
-      s_newdone[tid] = newdone;
-      s_bprev[tid] = bprev;
-      // the seed coefficient this launch's step uses (as ColRegs computes it), if it runs one
-      const float bnow = (mode == kStepRun && status == kColRunning)
-                             ? (float)((1.0 - (double)cr.damping) + (double)cr.damping * D)
-                             : bprev;
-      if (item.part == 0) {
-        if (mode == kStepFinish) {
-          PprCol* w = S->rec + tid;
-          w->status = status;
-          w->iters = iters;
-          w->dangling = D;
-          w->residual = res;
-          w->best = best;
-          w->stall = stall;
-          w->bused = bprev;
-        } else {
-          S->st[mode == kStepInit ? 0 : cur][tid] = ColState{status, iters, D, res, best, stall, bnow};
-        }
-      }
-    }
-    __syncthreads();
-
-    // ---- fresh columns start at e_seed (X and the current contributions)
-    if (mode == kStepInit) {
-      // one pass over the part's rows: every fresh column of a row at once;
-      // the other contribution buffer starts at 0 too (rows without in-edges
-      // are skipped by the steps: their x stays 0 unless seeded there)
-      T* Cc = (T*)S->C[S->parity];
-      T* Co = (T*)S->C[S->parity ^ 1];
-      const int k0 = 2 * lane, k1 = 2 * lane + 1;
-      const bool f0 = S->rec[k0].status == kColFresh, f1 = S->rec[k1].status == kColFresh;
-      const int32_t sr0 = s_seed[k0], sr1 = s_seed[k1];
-      if (__any_sync(0xffffffffu, f0 || f1)) {
-        for (int32_t p = r0 + warp; p < r1; p += kPprWarps) {
-          const float idg = inv_deg[p];
-          const int64_t o = (int64_t)p * kPprCols;
-          if (f0) {
-            const float v = p == sr0 ? 1.f : 0.f;
-            if (X) X[o + k0] = v;
-            st_one(Cc + o + k0, v * idg);
-            st_one(Co + o + k0, 0.f);
-          }
-          if (f1) {
-            const float v = p == sr1 ? 1.f : 0.f;
-            if (X) X[o + k1] = v;
-            st_one(Cc + o + k1, v * idg);
-            st_one(Co + o + k1, 0.f);
-          }
-          if (YS) {  // running sums 0; sent sums = the first delta (the whole contribution)
-            float4 r = YS[(int64_t)p * 32 + lane];
-            if (f0) {
-              r.x = 0.f;
-              r.z = p == sr0 ? bf16_bits_to_float(bf16_bits_rn(idg)) : 0.f;
-            }
-            if (f1) {
-              r.y = 0.f;
-              r.w = p == sr1 ? bf16_bits_to_float(bf16_bits_rn(idg)) : 0.f;
-            }
-            YS[(int64_t)p * 32 + lane] = r;
-          }
-        }
-      }
-      __syncthreads();
-    }
-
-    // ---- columns finished by now: this part's rows go out by node id, in
-    // one pass over the rows (a warp per row, two columns per lane)
-    {
-      const int k0 = 2 * lane, k1 = 2 * lane + 1;
-      const bool d0 = s_newdone[k0] != 0, d1 = s_newdone[k1] != 0;
-      if (__any_sync(0xffffffffu, d0 || d1)) {
-        float* o0 = d0 ? S->rec[k0].out : nullptr;
-        float* o1 = d1 ? S->rec[k1].out : nullptr;
-        const int64_t l0 = d0 ? S->rec[k0].ldo : 0, l1 = d1 ? S->rec[k1].ldo : 0;
-        for (int32_t p = r0 + warp; p < r1; p += kPprWarps) {
-          const int64_t v = S->new2old[p];
-          float2 x;
-          if (kDelta)  // x of the column's last step from its running sums
-            x = make_float2(x_from_ys(YS, p, k0, s_d[k0], s_seed[k0], s_bprev[k0]),
-                            x_from_ys(YS, p, k1, s_d[k1], s_seed[k1], s_bprev[k1]));
-          else
-            x = ld_state(X, p, lane);
-          if (d0) o0[v * l0] = x.x;
-          if (d1) o1[v * l1] = x.y;
-        }
-      }
-    }
-
-    if (mode == kStepRun) {
-      const T* __restrict__ Cin = (const T*)S->C[(S->parity + step - 1) & 1];
-      T* __restrict__ Cout = (T*)S->C[(S->parity + step) & 1];
-      const int32_t* __restrict__ col_ptr = S->col_ptr;
-      const int32_t* __restrict__ row_idx = S->row_idx;
-      ColRegs c;
-      {
-        const int k0 = 2 * lane, k1 = 2 * lane + 1;
-        c.l0 = s_status[k0] == kColRunning;
-        c.l1 = s_status[k1] == kColRunning;
-        c.a0 = s_d[k0];
-        c.a1 = s_d[k1];
-        c.b0 = (float)((1.0 - (double)s_d[k0]) + (double)s_d[k0] * s_D[k0]);
-        c.b1 = (float)((1.0 - (double)s_d[k1]) + (double)s_d[k1] * s_D[k1]);
-        c.s0 = s_seed[k0];
-        c.s1 = s_seed[k1];
-        c.bp0 = s_bprev[k0];
-        c.bp1 = s_bprev[k1];
-      }
-      float acc[2][3] = {{0.f, 0.f, 0.f}, {0.f, 0.f, 0.f}};
-      const int32_t heavy_deg = S->heavy_deg;
-      int32_t wr0, wr1;
-      warp_rows(col_ptr, r0, r1, warp, wr0, wr1);
-      // (a lane whose two columns are not running reads and writes nothing:
-      // a part-filled slot moves only the sectors of its running columns)
-      const bool on = c.l0 || c.l1;
-      for (int32_t p = wr0; p < wr1; ++p) {
-        const int32_t e0 = col_ptr[p], e1 = col_ptr[p + 1];
-        if (e1 - e0 > heavy_deg) continue;
-        // a row without in-edges keeps x = 0 (and contributions 0) unless it
-        // is a running column's seed
-        if (e0 == e1 && !__any_sync(0xffffffffu, (c.l0 && p == c.s0) || (c.l1 && p == c.s1))) continue;
-        const float2 xo = on && X ? ld_state(X, p, lane) : make_float2(0.f, 0.f);
-        const float4 ys = on ? ld_ys(YS, p, lane) : make_float4(0.f, 0.f, 0.f, 0.f);
-        const float2 y = gather_row(row_idx, Cin, e0, e1, lane, on);
-        if (on) finish_ppr_row(p, y, xo, ys, c, X, YS, Cout, inv_deg, lane, acc);
-      }
-      // long rows: their chunk sums (this step's chunk launch), in chunk
-      // order, a warp per row
-      const int32_t h0 = lower_bound_i32(S->heavy_rows, S->n_heavy, r0);
-      const int32_t h1 = lower_bound_i32(S->heavy_rows, S->n_heavy, r1);
-      for (int32_t hi = h0 + warp; on && hi < h1; hi += kPprWarps) {
-        const int32_t p = S->heavy_rows[hi];
-        const int32_t sp = S->heavy_split0 + hi;
-        float yx = 0.f, yy = 0.f;
-        for (int pass = 0; pass < 2; ++pass) {
-          const int32_t c0 = pass == 0 ? S->split_hbeg[sp] : S->split_cbeg[sp];
-          const int32_t c1 = pass == 0 ? S->split_hend[sp] : S->split_cend[sp];
-          for (int32_t c = c0; c < c1; ++c) {
-            const float2 v = __ldcg(reinterpret_cast<const float2*>(S->chunk_sum + (int64_t)c * kPprCols) + lane);
-            yx += v.x;
-            yy += v.y;
-          }
-        }
-        finish_ppr_row(p, make_float2(yx, yy), X ? ld_state(X, p, lane) : make_float2(0.f, 0.f), ld_ys(YS, p, lane),
-                       c, X, YS, Cout, inv_deg, lane, acc);
-      }
-      for (int v = 0; v < 3; ++v) {
-        s_wpart[warp][v][2 * lane] = acc[0][v];
-        s_wpart[warp][v][2 * lane + 1] = acc[1][v];
-      }
-      __syncthreads();
-      if (tid < 3 * kPprCols) {
-        const int v = tid / kPprCols, k = tid % kPprCols;
-        double sum = 0.0;
-        for (int w = 0; w < kPprWarps; ++w) sum += (double)s_wpart[w][v][k];
-        S->psum[cur][(3 * (int64_t)item.part + v) * kPprCols + k] = sum;
-      }
-    }
-    __syncthreads();  // shared state is reused by the next item
-  }
-}
-
-// Long-row chunk sums of one step: item (slot, q) covers chunks
-// [q * kChunksPerItem, (q + 1) * kChunksPerItem) of the slot's plan; a warp
-// gathers a chunk's edges for all 64 columns.
-template <typename T>
-__global__ void __launch_bounds__(kPprThreads, 1) ppr_chunk_kernel(const SlotDesc* __restrict__ slots,
-                                                                  const StepItem* __restrict__ items, int32_t nitems,
-                                                                  int32_t step) {
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  for (int32_t ii = blockIdx.x; ii < nitems; ii += gridDim.x) {
-    const StepItem item = items[ii];
-    const SlotDesc* S = slots + item.slot;
-    const T* __restrict__ Cin = (const T*)S->C[(S->parity + step - 1) & 1];
-    const int32_t c_end = min(S->nchunks, (item.part + 1) * kChunksPerItem);
-    // columns running after the previous step (the step launch may still stop
-    // some of them; their sums then go unused)
-    const ColState* stp = S->st[(step - 1) & 1];
-    const bool on = stp[2 * lane].status == kColRunning || stp[2 * lane + 1].status == kColRunning;
-    for (int32_t ch = item.part * kChunksPerItem + warp; ch < c_end; ch += kPprWarps) {
-      const float2 y = gather_row(S->row_idx, Cin, S->chunk_begin[ch], S->chunk_end[ch], lane, on);
-      reinterpret_cast<float2*>(S->chunk_sum + (int64_t)ch * kPprCols)[lane] = y;
-    }
-  }
-}
-
-__global__ void part_bounds_kernel(const int32_t* __restrict__ col_ptr, int32_t n, int64_t m, int32_t nparts,
-                                   int32_t* __restrict__ part_rows) {
-  for (int32_t i = blockIdx.x * blockDim.x + threadIdx.x; i <= nparts; i += gridDim.x * blockDim.x) {
-    if (i == 0) {
-      part_rows[i] = 0;
-    } else if (i == nparts) {
-      part_rows[i] = n;
-    } else {
-      const int64_t work = m + kRowWeight * n;  // edges + kRowWeight * rows
-      const int64_t target = (work * i + nparts - 1) / nparts;
-      part_rows[i] = min(n, lower_bound_work(col_ptr, n, target));
-    }
-  }
-}
-
 // ---- host side ----------------------------------------------------------------
-
-void heavy_of(const gpr_graph* g, const int32_t** rows, int32_t* n, int32_t* deg, int32_t* split0) {
-  const Plan& P = g->plan;
-  *rows = P.rows;
-  *n = 0;
-  *deg = INT_MAX;
-  *split0 = 0;
-  // the long rows are the last chunked (lanes 0) bucket; the plan's split
-  // entries list the rows of every chunked bucket in bucket order
-  int32_t before = 0;
-  for (int b = 0; b < P.nbuckets; ++b)
-    if (P.bucket[b].lanes == 0) {
-      *split0 = before;
-      *rows = P.rows + P.bucket[b].row_begin;
-      *n = P.bucket[b].row_end - P.bucket[b].row_begin;
-      *deg = b > 0 ? P.deg_threshold[b - 1] : -1;  // bucket 0 holds every degree from 0
-      before += *n;
-    }
-}
 
 template <typename T>
 static int max_clusters_for(int cluster) {
@@ -861,56 +518,6 @@ static int max_clusters_for(int cluster) {
   }
   return num;
 }
-
-void ppr_part_bounds(const int32_t* col_ptr, int32_t n, int64_t m, int32_t nparts, int32_t* part_rows,
-                     cudaStream_t s) {
-  part_bounds_kernel<<<std::max(1, (nparts + 256) / 256), 256, 0, s>>>(col_ptr, n, m, nparts, part_rows);
-  GPR_CUDA(cudaGetLastError());
-  count_launches(1);
-}
-
-template <typename T>
-static int step_grid(int32_t nitems) {
-  int per_sm = 0;
-  cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, ppr_step_kernel<T>, kPprThreads, 0);
-  return std::max(1, std::min(nitems, num_sms() * std::max(per_sm, 1)));
-}
-
-void ppr_step_launch(const SlotDesc* slots_dev, const StepItem* items_dev, int32_t nitems, int mode, int32_t step,
-                     gpr_dtype dt, cudaStream_t s) {
-  if (nitems <= 0) return;
-  if (dt == GPR_BF16)
-    ppr_step_kernel<__nv_bfloat16><<<step_grid<__nv_bfloat16>(nitems), kPprThreads, 0, s>>>(slots_dev, items_dev,
-                                                                                          nitems, mode, step);
-  else if (dt == GPR_FP16)
-    ppr_step_kernel<__half><<<step_grid<__half>(nitems), kPprThreads, 0, s>>>(slots_dev, items_dev, nitems, mode, step);
-  else
-    ppr_step_kernel<float><<<step_grid<float>(nitems), kPprThreads, 0, s>>>(slots_dev, items_dev, nitems, mode, step);
-  GPR_CUDA(cudaGetLastError());
-  count_launches(1);
-}
-
-template <typename T>
-static int chunk_grid(int32_t nitems) {
-  int per_sm = 0;
-  cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, ppr_chunk_kernel<T>, kPprThreads, 0);
-  return std::max(1, std::min(nitems, num_sms() * std::max(per_sm, 1)));
-}
-
-void ppr_chunk_launch(const SlotDesc* slots_dev, const StepItem* items_dev, int32_t nitems, int32_t step,
-                      gpr_dtype dt, cudaStream_t s) {
-  if (nitems <= 0) return;
-  if (dt == GPR_BF16)
-    ppr_chunk_kernel<__nv_bfloat16><<<chunk_grid<__nv_bfloat16>(nitems), kPprThreads, 0, s>>>(slots_dev, items_dev,
-                                                                                            nitems, step);
-  else if (dt == GPR_FP16)
-    ppr_chunk_kernel<__half><<<chunk_grid<__half>(nitems), kPprThreads, 0, s>>>(slots_dev, items_dev, nitems, step);
-  else
-    ppr_chunk_kernel<float><<<chunk_grid<float>(nitems), kPprThreads, 0, s>>>(slots_dev, items_dev, nitems, step);
-  GPR_CUDA(cudaGetLastError());
-  count_launches(1);
-}
-
 
 static int max_clusters(gpr_dtype dt, int cluster) {
   if (dt == GPR_BF16) return max_clusters_for<__nv_bfloat16>(cluster);

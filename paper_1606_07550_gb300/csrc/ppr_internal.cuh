@@ -1,5 +1,5 @@
 // Device-side records of the batched personalised-PageRank kernel, shared by
-// the one-shot batch call (ppr.cu) and the continuous-batching server
+// the one-shot batch call (ppr.cu, ppr_steps.cu) and the continuous-batching server
 // (serve.cu).
 #pragma once
 
@@ -55,70 +55,78 @@ struct PprJob {
   PprCol* cols;         // 64 records
 };
 
-// ---- step-major execution for the server --------------------------------
-// A slot's rows are split into parts of about equal edge count; one launch
-// runs one step of every (slot, part) item, so a large graph is spread over
-// every SM.  The per-column sums of a step are folded, in part order, at the
-// start of the next launch; column state is double-buffered by step parity.
-struct ColState {
-  int32_t status, iters;
-  double dangling, residual, best;
-  int32_t stall;
-  float bused;  // seed coefficient used by the step of the launch that wrote this state (1 before the first)
-};
+// ---- step-major execution (ppr_steps.cu) --------------------------------------
+constexpr int kStWarps = 8;          // warps of a block
+constexpr int64_t kPieceWork = 256;  // work of a piece: an edge counts 1, a row 3
 
-struct SlotDesc {
+struct StepState;
+
+// One graph with up to 64 columns: a job of a batch, or a slot of the server.
+struct StepJob {
   const int32_t* col_ptr;
   const int32_t* row_idx;
   const float* inv_deg;
   const int32_t* old2new;
   const int32_t* new2old;
+  int64_t m;
+  int32_t n, npieces, nitems;
+  int32_t per;          // pieces of an item for each of its block's warps
+  int32_t long_deg;     // rows of more edges are summed by chunks
+  int32_t* prows;       // npieces + 1 row boundaries
+  int32_t* long_base;   // a batch's: first chunk of each long row (n entries)
+  float* X;             // n x W: x, or with BF16 deltas the running sums
+  void* C[2];           // (n + 1) x W: contributions, and a row of zeros
+  float* S;             // n x W: sent sums (BF16 deltas)
+  float* chunk_sum;     // chunks x W
+  // a slot's long rows and chunks are the graph plan's: long row i of
+  // heavy_rows (ascending) sums chunks [hbeg, hend) then [cbeg, cend) of split
+  // entry split0 + i
   const int32_t* heavy_rows;
-  int32_t n_heavy, heavy_deg;
-  int32_t n, nparts;
-  const int32_t* part_rows;  // nparts + 1 row boundaries
-  float* X;
-  void* C[2];
-  float4* YS;                // BF16 deltas: per row and lane the running and sent sums (null otherwise)
-  int32_t parity;            // C buffer holding the contributions at the start of the tick
-  int32_t pad;
-  PprCol* rec;               // 64 host-visible records
-  ColState* st[2];           // 64 each, by step parity
-  double* psum[2];           // nparts x 3 x 64 each, by step parity
-  // long rows (heavy_rows) as edge chunks of the graph's plan: long row i
-  // sums chunks [hbeg, hend) then [cbeg, cend) of split entry heavy_split0 + i
   const int32_t* chunk_begin;
   const int32_t* chunk_end;
   const int32_t* split_hbeg;
   const int32_t* split_hend;
   const int32_t* split_cbeg;
   const int32_t* split_cend;
-  int32_t nchunks, heavy_split0;
-  float* chunk_sum;          // nchunks x 64: the chunk's sums of this step
+  int32_t n_heavy, split0, nchunks;
+  int32_t parity;       // C[parity & 1] holds the contributions before step 0
+  StepState* st;
+  PprCol* cols;         // 64 records
+};
+
+// The state of a job's columns between two steps.
+struct StepState {
+  float d[kPprCols], b[kPprCols], bprev[kPprCols], tol[kPprCols];
+  int32_t seed[kPprCols], status[kPprCols], iters[kPprCols], stall[kPprCols], max_iters[kPprCols];
+  double res[kPprCols], best[kPprCols];
+  unsigned long long acc[2][kPprCols];  // this step's dangling masses and residuals so far
+  uint32_t arrived;                     // items that have added theirs
+  int32_t live;                         // columns still running
+};
+
+// A chunk of a long row: edges [e0, e1) of job `slot`.
+struct LongChunk {
+  int32_t slot, e0, e1, pad;
 };
 
 struct StepItem {
   int32_t slot, part;
 };
 
-// 64 consecutive long-row chunks of one slot.
-constexpr int32_t kChunksPerItem = 64;
-
-enum : int { kStepInit = 0, kStepRun = 1, kStepFinish = 2 };
-
-void ppr_step_launch(const SlotDesc* slots_dev, const StepItem* items_dev, int32_t nitems, int mode, int32_t step,
-                     gpr_dtype dt, cudaStream_t s);
-// The long-row chunk sums of step `step` for chunk items (slot, first chunk / kChunksPerItem).
-void ppr_chunk_launch(const SlotDesc* slots_dev, const StepItem* items_dev, int32_t nitems, int32_t step,
-                      gpr_dtype dt, cudaStream_t s);
-void ppr_part_bounds(const int32_t* col_ptr, int32_t n, int64_t m, int32_t nparts, int32_t* part_rows,
-                     cudaStream_t s);
-
+// Pieces of g's rows, of about kPieceWork work each.
+int32_t ppr_pieces(const gpr_graph* g);
+// The pieces' row boundaries (ppr_pieces(g) + 1).
+void ppr_piece_bounds(const gpr_graph* g, int32_t* prows, cudaStream_t s);
 // The long rows of g's plan (in-degree above *deg): *n ascending row ids, the
 // first of them split entry *split0 of the plan's chunk lists.
 void heavy_of(const gpr_graph* g, const int32_t** rows, int32_t* n, int32_t* deg, int32_t* split0);
+// `steps` steps of the slots of `items`, (slot, q) for every kStWarps x per pieces:
+// columns with status kColFresh in their records join first,
+// finished ones go out by node id at the end, when the records are written.
+// citems: (slot, q) for every kStWarps chunks of the slots.  scratch: a word.
+void ppr_slot_steps(const StepJob* jobs, const StepItem* items, int nitems, const StepItem* citems, int ncitems,
+                    int32_t steps, gpr_dtype dt, uint32_t* scratch, cudaStream_t s);
 
-// ---- step-major execution of a batch (ppr_steps.cu) ------------------------
 // One graph with k <= 64 columns, whose 64 records are in device memory: the
 // outputs of columns 0..k-1 are consecutive floats of a row of x_out.
 struct StepRequest {

@@ -47,6 +47,9 @@
 // the short rows (up to kShortDeg edges) before the others, each in row order;
 // then exact integer sums of those in units of 2^-kFixBits, in any order.
 //
+// The server (serve.cu) runs its slots' steps on the same kernels, 64 columns
+// wide.
+//
 // Storage of the contributions as in ppr.cu: FP32; FP16 times 2^10; BF16 as
 // error-feedback deltas (X then holds the running sums y, S the sent ones).
 #include <algorithm>
@@ -61,51 +64,15 @@
 
 namespace gpr {
 
-constexpr int kStThreads = 256;
-constexpr int kStWarps = kStThreads / 32;
-constexpr int64_t kPieceWork = 256;  // work of a piece: an edge counts 1, a row 3
-constexpr int32_t kLongDeg = 128;    // longer rows are summed by chunks
+constexpr int kStThreads = 32 * kStWarps;
+constexpr int32_t kLongDeg = 128;    // a batch's longer rows are summed by chunks
 constexpr int32_t kShortDeg = 8;     // rows that half a warp takes
 constexpr int kFixBits = 60;         // dangling masses and residuals are sums of multiples of 2^-60, below 8
 
-// One job of a wave.
-struct StepJob {
-  const int32_t* col_ptr;
-  const int32_t* row_idx;
-  const float* inv_deg;
-  const int32_t* old2new;
-  const int32_t* new2old;
-  int32_t n, k, npieces, nitems;
-  int64_t m;
-  int32_t* prows;     // npieces + 1 row boundaries
-  int32_t* long_base; // n: first chunk of a long row
-  float* X;           // n x W: x, or with BF16 deltas the running sums
-  void* C[2];         // (n + 1) x W: contributions, and a row of zeros
-  float* S;           // n x W: sent sums (BF16 deltas)
-  struct StepState* st;
-  PprCol* cols;       // 64 records
-  int32_t max_iters, pad;
-};
-
-// The state of a job's columns between two steps.
-struct StepState {
-  float d[kPprCols], b[kPprCols], bprev[kPprCols], tol[kPprCols];
-  int32_t seed[kPprCols], status[kPprCols], iters[kPprCols], stall[kPprCols];
-  double res[kPprCols], best[kPprCols];
-  unsigned long long acc[2][kPprCols];  // this step's dangling masses and residuals so far
-  uint32_t arrived;                     // items that have added theirs
-  int32_t live;                         // columns still running
-};
-
-// A chunk of a long row: edges [e0, e1) of job `slot`.
-struct LongChunk {
-  int32_t slot, e0, e1, pad;
-};
-
-// Edges per chunk of a row of deg edges: about sqrt(2 deg), since the chunk
-// sums of one row are added by one warp.
-__host__ __device__ __forceinline__ int32_t chunk_edges(int32_t deg) {
-  int32_t c = kLongDeg;
+// Edges per chunk of a row of deg edges, more than long_deg: long_deg, or about
+// sqrt(2 deg), since the chunk sums of one row are added by one warp.
+__host__ __device__ __forceinline__ int32_t chunk_edges(int32_t deg, int32_t long_deg) {
+  int32_t c = long_deg;
   while (deg / c >= 2 * c) c *= 2;
   return c;
 }
@@ -489,10 +456,10 @@ __device__ __forceinline__ void finish_cols(int32_t p, const float (&y)[Geo<W>::
 
 // The sum of a long row's chunk sums, in order.
 template <int W>
-__device__ __forceinline__ void sum_chunks(const float* __restrict__ chunk_sum, int32_t first, int32_t deg, int c0,
-                                           float (&y)[Geo<W>::V]) {
+__device__ __forceinline__ void sum_chunks(const float* __restrict__ chunk_sum, int32_t first, int32_t deg,
+                                           int32_t long_deg, int c0, float (&y)[Geo<W>::V]) {
   constexpr int V = Geo<W>::V;
-  const int32_t c = chunk_edges(deg), cnt = (deg + c - 1) / c;
+  const int32_t c = chunk_edges(deg, long_deg), cnt = (deg + c - 1) / c;
   const float* base = chunk_sum + (int64_t)first * W + c0;
 #pragma unroll
   for (int v = 0; v < V; ++v) y[v] = 0.f;
@@ -514,12 +481,40 @@ __device__ __forceinline__ void sum_chunks(const float* __restrict__ chunk_sum, 
   }
 }
 
+// The same of a slot's long row p, from the plan's chunks.
+template <int W>
+__device__ __forceinline__ void sum_plan_chunks(const StepJob* J, int32_t p, int c0, float (&y)[Geo<W>::V]) {
+  constexpr int V = Geo<W>::V;
+  int32_t lo = 0, hi = J->n_heavy;  // p's place among the long rows
+  while (hi - lo > 1) {
+    const int32_t mid = lo + (hi - lo) / 2;
+    if (J->heavy_rows[mid] <= p)
+      lo = mid;
+    else
+      hi = mid;
+  }
+  const int32_t sp = J->split0 + lo;
+#pragma unroll
+  for (int v = 0; v < V; ++v) y[v] = 0.f;
+  for (int pass = 0; pass < 2; ++pass) {
+    const int32_t k0 = pass == 0 ? J->split_hbeg[sp] : J->split_cbeg[sp];
+    const int32_t k1 = pass == 0 ? J->split_hend[sp] : J->split_cend[sp];
+#pragma unroll 4
+    for (int32_t k = k0; k < k1; ++k) {
+      float z[V];
+      ld_c<V>((const float*)J->chunk_sum + (int64_t)k * W + c0, z);
+#pragma unroll
+      for (int v = 0; v < V; ++v) y[v] += z[v];
+    }
+  }
+}
+
 // One step of every item: item (job, q) takes the pieces
 // [q * per, (q + 1) * per) * kStWarps of its job, its warps one after another.
-template <typename T, int W>
+// kSlot: a slot of the server (its long rows' chunks are the plan's).
+template <typename T, int W, bool kSlot>
 __global__ void __launch_bounds__(kStThreads, 3) ppr_rows_kernel(const StepJob* __restrict__ jobs,
-                                                             const StepItem* __restrict__ items, int per, int parity,
-                                                             const float* __restrict__ chunk_sum,
+                                                             const StepItem* __restrict__ items, int step,
                                                              uint32_t* __restrict__ live_jobs) {
   constexpr int V = Geo<W>::V, L = Geo<W>::L, R = Geo<W>::R;
   __shared__ ColShared<W> cs;
@@ -544,9 +539,13 @@ __global__ void __launch_bounds__(kStThreads, 3) ppr_rows_kernel(const StepJob* 
   const int32_t* __restrict__ col_ptr = J->col_ptr;
   const int32_t* __restrict__ row_idx = J->row_idx;
   const int32_t* __restrict__ prows = J->prows;
+  const int parity = (J->parity + step) & 1;
   const T* __restrict__ Cin = (const T*)J->C[parity];
   T* __restrict__ Cout = (T*)J->C[parity ^ 1];
-  const int32_t piece0 = item.part * kStWarps * per, pieces = min(kStWarps * per, J->npieces - piece0);
+  const float* __restrict__ chunk_sum = J->chunk_sum;
+  int32_t long_deg = kLongDeg;
+  if constexpr (kSlot) long_deg = J->long_deg;
+  const int32_t per = J->per, piece0 = item.part * kStWarps * per, pieces = min(kStWarps * per, J->npieces - piece0);
   if (tid == 0) s_next = kStWarps;
   __syncthreads();
   const int c0 = (lane % L) * V;
@@ -643,7 +642,7 @@ __global__ void __launch_bounds__(kStThreads, 3) ppr_rows_kernel(const StepJob* 
           nrow = base + b;
           ne0 = __shfl_sync(0xffffffffu, e0, b);
           ne1 = __shfl_sync(0xffffffffu, e1, b);
-          nidx = ne0 + lane < ne1 && ne1 - ne0 <= kLongDeg ? __ldcs(row_idx + ne0 + lane) : n;
+          nidx = ne0 + lane < ne1 && ne1 - ne0 <= long_deg ? __ldcs(row_idx + ne0 + lane) : n;
         };
         if (W == 64) shorts = 0;
         bool more = (shorts | others) != 0;
@@ -654,9 +653,12 @@ __global__ void __launch_bounds__(kStThreads, 3) ppr_rows_kernel(const StepJob* 
           more = (shorts | others) != 0;
           if (more) ahead();
           float y[V];
-          if (a1 - a0 > kLongDeg)
-            sum_chunks<W>(chunk_sum, J->long_base[row], a1 - a0, c0, y);
-          else
+          if (a1 - a0 > long_deg) {
+            if constexpr (kSlot)
+              sum_plan_chunks<W>(J, row, c0, y);
+            else
+              sum_chunks<W>(chunk_sum, J->long_base[row], a1 - a0, long_deg, c0, y);
+          } else
             gather_warp_row<T, W>(row_idx, cbase, stride, n, a0, a1, idx, lane, y);
           if (on) {
             float dn[V], rs[V];
@@ -701,8 +703,8 @@ __global__ void __launch_bounds__(kStThreads, 3) ppr_rows_kernel(const StepJob* 
           float y[V];
           const int32_t deg = a1 - a0;
           gather_narrow_short<T, W>(row_idx, Cin, a0, deg <= 64 ? a1 : a0, u, lane, y);
-          if (deg > kLongDeg) sum_chunks<W>(chunk_sum, J->long_base[row], deg, c0, y);
-          uint32_t lm = __ballot_sync(0xffffffffu, deg > 64 && deg <= kLongDeg) & 0x01010101u;  // a lane of each
+          if (deg > long_deg) sum_chunks<W>(chunk_sum, J->long_base[row], deg, long_deg, c0, y);
+          uint32_t lm = __ballot_sync(0xffffffffu, deg > 64 && deg <= long_deg) & 0x01010101u;  // a lane of each
           while (lm) {
             const int src = __ffs(lm) - 1;
             lm &= lm - 1;
@@ -768,7 +770,7 @@ __global__ void __launch_bounds__(kStThreads, 3) ppr_rows_kernel(const StepJob* 
     }
     const float tol = st->tol[tid];
     const bool stop = (tol > 0.f && ((d / (1.0 - d)) * res <= (double)tol || stall >= kStallSteps)) ||
-                      it >= J->max_iters;
+                      it >= st->max_iters[tid];
     st->bprev[tid] = cs.b[tid];
     st->b[tid] = (float)((1.0 - d) + d * D);
     st->res[tid] = res;
@@ -785,56 +787,100 @@ __global__ void __launch_bounds__(kStThreads, 3) ppr_rows_kernel(const StepJob* 
   }
 }
 
-// The chunk sums of the long rows of a wave, a warp per chunk.
+// The sum of one chunk of a long row, a warp's work.
+template <typename T, int W>
+__device__ __forceinline__ void long_chunk(const StepJob* J, int32_t e0, int32_t e1, int32_t ch, int step, int lane) {
+  constexpr int V = Geo<W>::V, L = Geo<W>::L, R = Geo<W>::R;
+  const StepState* st = J->st;
+  if (st->live == 0) return;
+  const int c0 = (lane % L) * V;
+  bool on = false;
+#pragma unroll
+  for (int v = 0; v < V; ++v) on = on || st->status[c0 + v] == kColRunning;
+  const T* __restrict__ Cin = (const T*)J->C[(J->parity + step) & 1];
+  float y[V];
+  if constexpr (R == 1) {
+    const int32_t n = J->n;
+    const int32_t idx = e0 + lane < e1 ? __ldcs(J->row_idx + e0 + lane) : n;
+    gather_warp_row<T, W>(J->row_idx, Cin + c0 + (on ? 0 : (int64_t)n * W), on ? W : 0, n, e0, e1, idx, lane, y);
+  } else {
+    gather_narrow_long<T, W>(J->row_idx, Cin, e0, e1, lane, y);
+  }
+  if (on && lane < L) st_c<V>(J->chunk_sum + (int64_t)ch * W + c0, y);
+}
+
+// The chunk sums of the long rows of a batch's wave, a warp per chunk of its
+// list.
 template <typename T, int W>
 __global__ void __launch_bounds__(kStThreads) ppr_long_kernel(const StepJob* __restrict__ jobs,
                                                              const LongChunk* __restrict__ chunks,
-                                                             const int32_t* __restrict__ nchunks, int parity,
-                                                             float* __restrict__ chunk_sum) {
-  constexpr int V = Geo<W>::V, L = Geo<W>::L, R = Geo<W>::R;
-  const int lane = threadIdx.x & 31;
+                                                             const int32_t* __restrict__ nchunks, int step) {
   const int32_t total = *nchunks;
   for (int32_t ch = blockIdx.x * kStWarps + (threadIdx.x >> 5); ch < total; ch += gridDim.x * kStWarps) {
     const LongChunk lc = chunks[ch];
-    const StepJob* J = jobs + lc.slot;
-    const StepState* st = J->st;
-    if (st->live == 0) continue;
-    const int c0 = (lane % L) * V;
-    bool on = false;
-#pragma unroll
-    for (int v = 0; v < V; ++v) on = on || st->status[c0 + v] == kColRunning;
-    const T* __restrict__ Cin = (const T*)J->C[parity];
-    float y[V];
-    if constexpr (R == 1) {
-      const int32_t n = J->n;
-      const int32_t idx = lc.e0 + lane < lc.e1 ? __ldcs(J->row_idx + lc.e0 + lane) : n;
-      gather_warp_row<T, W>(J->row_idx, Cin + c0 + (on ? 0 : (int64_t)n * W), on ? W : 0, n, lc.e0, lc.e1, idx, lane,
-                            y);
-    } else {
-      gather_narrow_long<T, W>(J->row_idx, Cin, lc.e0, lc.e1, lane, y);
-    }
-    if (on && lane < L) st_c<V>(chunk_sum + (int64_t)ch * W + c0, y);
+    long_chunk<T, W>(jobs + lc.slot, lc.e0, lc.e1, ch, step, threadIdx.x & 31);
   }
 }
 
+// The same of the server's slots: item (slot, q) takes the slot's chunks
+// [q * kStWarps, (q + 1) * kStWarps).
+template <typename T>
+__global__ void __launch_bounds__(kStThreads) ppr_slot_long_kernel(const StepJob* __restrict__ jobs,
+                                                                  const StepItem* __restrict__ items, int step) {
+  const StepItem item = items[blockIdx.x];
+  const StepJob* J = jobs + item.slot;
+  const int32_t ch = item.part * kStWarps + (threadIdx.x >> 5);
+  if (ch >= J->nchunks) return;
+  long_chunk<T, kPprCols>(J, J->chunk_begin[ch], J->chunk_end[ch], ch, step, threadIdx.x & 31);
+}
+
 // Row boundaries of a job's pieces: equal shares of edges + 3 * rows.
-__global__ void ppr_bounds_kernel(const StepJob* __restrict__ jobs) {
-  const StepJob* J = jobs + blockIdx.y;
-  const int32_t cnt = J->npieces;
-  const int64_t work = J->m + 3 * (int64_t)J->n;
+__device__ __forceinline__ void piece_bounds(const int32_t* __restrict__ col_ptr, int32_t n, int64_t m, int32_t cnt,
+                                             int32_t* __restrict__ prows) {
+  const int64_t work = m + 3 * (int64_t)n;
   for (int32_t i = blockIdx.x * blockDim.x + threadIdx.x; i <= cnt; i += gridDim.x * blockDim.x) {
     const int64_t key = (work * i + cnt - 1) / cnt;
-    int32_t lo = 0, hi = J->n;
+    int32_t lo = 0, hi = n;
     if (i == cnt) lo = hi;
     while (lo < hi) {
       const int32_t mid = lo + (hi - lo) / 2;
-      if ((int64_t)J->col_ptr[mid] + 3 * (int64_t)mid < key)
+      if ((int64_t)col_ptr[mid] + 3 * (int64_t)mid < key)
         lo = mid + 1;
       else
         hi = mid;
     }
-    J->prows[i] = lo;
+    prows[i] = lo;
   }
+}
+__global__ void ppr_bounds_kernel(const StepJob* __restrict__ jobs) {
+  const StepJob* J = jobs + blockIdx.y;
+  piece_bounds(J->col_ptr, J->n, J->m, J->npieces, J->prows);
+}
+
+__global__ void ppr_graph_bounds_kernel(const int32_t* __restrict__ col_ptr, int32_t n, int64_t m, int32_t cnt,
+                                        int32_t* __restrict__ prows) {
+  piece_bounds(col_ptr, n, m, cnt, prows);
+}
+
+// Column k starts from its record; returns whether it has a step to run.
+__device__ __forceinline__ int start_column(const StepJob* J, const PprCol& c, int k) {
+  StepState* st = J->st;
+  const int32_t seed = J->old2new[c.seed];
+  const double d = c.damping, D = J->inv_deg[seed] == 0.f ? 1.0 : 0.0;
+  const int live = c.max_iters > 0;
+  st->d[k] = c.damping;
+  st->b[k] = (float)((1.0 - d) + d * D);
+  st->bprev[k] = 1.f;  // x_0 = e_seed
+  st->tol[k] = c.tol;
+  st->max_iters[k] = c.max_iters;
+  st->seed[k] = seed;
+  st->status[k] = live ? kColRunning : kColDone;
+  st->iters[k] = 0;
+  st->stall[k] = 0;
+  st->res[k] = 0.0;
+  st->best[k] = INFINITY;
+  st->acc[0][k] = st->acc[1][k] = 0ull;
+  return live;
 }
 
 // x_0 = e_seed: the state and contributions of a job's rows (item by item),
@@ -843,7 +889,7 @@ __global__ void ppr_bounds_kernel(const StepJob* __restrict__ jobs) {
 // of its columns.
 template <typename T, int W>
 __global__ void __launch_bounds__(kStThreads) ppr_start_kernel(const StepJob* __restrict__ jobs,
-                                                              const StepItem* __restrict__ items, int per,
+                                                              const StepItem* __restrict__ items,
                                                               LongChunk* __restrict__ chunks,
                                                               int32_t* __restrict__ nchunks,
                                                               uint32_t* __restrict__ live_jobs) {
@@ -861,21 +907,10 @@ __global__ void __launch_bounds__(kStThreads) ppr_start_kernel(const StepJob* __
     int live = 0;
     if (tid < kPprCols) {
       const PprCol c = J->cols[tid];
-      const bool fresh = tid < W && c.status == kColFresh;
-      const int32_t seed = fresh ? J->old2new[c.seed] : -1;
-      const double d = c.damping, D = fresh && J->inv_deg[seed] == 0.f ? 1.0 : 0.0;
-      live = fresh && J->max_iters > 0;
-      st->d[tid] = c.damping;
-      st->b[tid] = (float)((1.0 - d) + d * D);
-      st->bprev[tid] = 1.f;  // x_0 = e_seed
-      st->tol[tid] = c.tol;
-      st->seed[tid] = seed;
-      st->status[tid] = live ? kColRunning : fresh ? kColDone : kColEmpty;
-      st->iters[tid] = 0;
-      st->stall[tid] = 0;
-      st->res[tid] = 0.0;
-      st->best[tid] = INFINITY;
-      st->acc[0][tid] = st->acc[1][tid] = 0ull;
+      if (tid < W && c.status == kColFresh)
+        live = start_column(J, c, tid);
+      else
+        st->status[tid] = kColEmpty;
     }
     live = __syncthreads_count(live);
     if (tid == 0) {
@@ -885,12 +920,12 @@ __global__ void __launch_bounds__(kStThreads) ppr_start_kernel(const StepJob* __
     }
   }
   __syncthreads();
-  const int32_t piece0 = min(item.part * kStWarps * per, J->npieces);
+  const int32_t per = J->per, piece0 = min(item.part * kStWarps * per, J->npieces);
   const int32_t r0 = J->prows[piece0], r1 = J->prows[min(piece0 + kStWarps * per, J->npieces)];
   for (int32_t p = r0 + tid; p < r1; p += kStThreads) {
     const int32_t e0 = J->col_ptr[p], deg = J->col_ptr[p + 1] - e0;
     if (deg <= kLongDeg) continue;
-    const int32_t c = chunk_edges(deg), cnt = (deg + c - 1) / c, first = atomicAdd(nchunks, cnt);
+    const int32_t c = chunk_edges(deg, kLongDeg), cnt = (deg + c - 1) / c, first = atomicAdd(nchunks, cnt);
     J->long_base[p] = first;
     for (int32_t k = 0; k < cnt; ++k)
       chunks[first + k] = LongChunk{item.slot, e0 + k * c, e0 + min(deg, (k + 1) * c), 0};
@@ -922,40 +957,108 @@ __global__ void __launch_bounds__(kStThreads) ppr_start_kernel(const StepJob* __
   }
 }
 
-// The finished columns by node id, and their records.
-template <typename T, int W>
-__global__ void __launch_bounds__(kStThreads) ppr_out_kernel(const StepJob* __restrict__ jobs,
-                                                            const StepItem* __restrict__ items, int per) {
+// The same for the columns that have joined a server's slot (status kColFresh
+// in its records) since its last steps; those that finished then leave.
+template <typename T>
+__global__ void __launch_bounds__(kStThreads) ppr_join_kernel(const StepJob* __restrict__ jobs,
+                                                             const StepItem* __restrict__ items) {
   constexpr bool kDelta = std::is_same<T, __nv_bfloat16>::value;
-  __shared__ float s_d[W], s_b[W];
+  constexpr int W = kPprCols;
   __shared__ int32_t s_seed[W];
+  __shared__ uint8_t s_fresh[W];
   const StepItem item = items[blockIdx.x];
   const StepJob* J = jobs + item.slot;
-  const StepState* st = J->st;
   const int tid = threadIdx.x;
+  int fresh = 0;
   if (tid < W) {
-    s_d[tid] = st->d[tid];
-    s_b[tid] = st->bprev[tid];
-    s_seed[tid] = st->seed[tid];
+    const PprCol c = J->cols[tid];
+    fresh = c.status == kColFresh;
+    s_fresh[tid] = (uint8_t)fresh;
+    s_seed[tid] = fresh ? J->old2new[c.seed] : -1;
   }
-  __syncthreads();
-  if (item.part == 0 && tid < W) {
-    PprCol* c = J->cols + tid;
-    c->status = st->status[tid];
-    c->iters = st->iters[tid];
-    c->residual = st->res[tid];
+  if (item.part == 0) {
+    StepState* st = J->st;
+    int live = 0;
+    if (tid < W) {
+      if (fresh)
+        live = start_column(J, J->cols[tid], tid);
+      else if (st->status[tid] == kColRunning)
+        live = 1;
+      else
+        st->status[tid] = kColEmpty;
+    }
+    live = __syncthreads_count(live);
+    if (tid == 0) {
+      st->arrived = 0;
+      st->live = live;
+    }
   }
-  float* out = J->cols[0].out;  // the job's columns are consecutive
-  const int64_t ldo = J->cols[0].ldo;
-  const int32_t piece0 = min(item.part * kStWarps * per, J->npieces);
+  if (!__syncthreads_or(fresh)) return;
+  const int parity = J->parity & 1;
+  T* Cc = (T*)J->C[parity];
+  T* Co = (T*)J->C[parity ^ 1];
+  const int32_t per = J->per, piece0 = min(item.part * kStWarps * per, J->npieces);
   const int64_t i0 = (int64_t)J->prows[piece0] * W;
   const int64_t i1 = (int64_t)J->prows[min(piece0 + kStWarps * per, J->npieces)] * W;
   for (int64_t i = i0 + tid; i < i1; i += kStThreads) {
     const int32_t p = (int32_t)(i / W), k = (int32_t)(i % W);
-    if (k >= J->k) continue;
+    if (!s_fresh[k]) continue;
+    float x = 0.f, c[1] = {0.f};
+    if (s_seed[k] == p) {
+      x = 1.f;
+      c[0] = J->inv_deg[p];
+    }
+    if (kDelta) {
+      J->X[i] = 0.f;
+      J->S[i] = __bfloat162float(__float2bfloat16_rn(c[0]));
+    } else {
+      J->X[i] = x;
+    }
+    st_c<1>(Cc + i, c);
+    c[0] = 0.f;
+    st_c<1>(Co + i, c);
+  }
+}
+
+// The finished columns by node id, and the records of all.
+template <typename T, int W>
+__global__ void __launch_bounds__(kStThreads) ppr_out_kernel(const StepJob* __restrict__ jobs,
+                                                            const StepItem* __restrict__ items) {
+  constexpr bool kDelta = std::is_same<T, __nv_bfloat16>::value;
+  __shared__ float s_d[W], s_b[W];
+  __shared__ int32_t s_seed[W], s_ldo[W];
+  __shared__ float* s_out[W];  // null: not finished
+  const StepItem item = items[blockIdx.x];
+  const StepJob* J = jobs + item.slot;
+  const StepState* st = J->st;
+  const int tid = threadIdx.x;
+  int done = 0;
+  if (tid < W) {
+    const int32_t status = st->status[tid];
+    done = status == kColDone;
+    s_d[tid] = st->d[tid];
+    s_b[tid] = st->bprev[tid];
+    s_seed[tid] = st->seed[tid];
+    PprCol* c = J->cols + tid;
+    s_out[tid] = done ? c->out : nullptr;
+    s_ldo[tid] = c->ldo;
+    if (item.part == 0 && status != kColEmpty) {
+      c->status = status;
+      c->iters = st->iters[tid];
+      c->residual = st->res[tid];
+    }
+  }
+  if (!__syncthreads_or(done)) return;
+  const int32_t per = J->per, piece0 = min(item.part * kStWarps * per, J->npieces);
+  const int64_t i0 = (int64_t)J->prows[piece0] * W;
+  const int64_t i1 = (int64_t)J->prows[min(piece0 + kStWarps * per, J->npieces)] * W;
+  for (int64_t i = i0 + tid; i < i1; i += kStThreads) {
+    const int32_t p = (int32_t)(i / W), k = (int32_t)(i % W);
+    float* out = s_out[k];
+    if (!out) continue;
     float x = __ldcs(J->X + i);
     if (kDelta) x = fmaf(s_d[k], x, p == s_seed[k] ? s_b[k] : 0.f);
-    out[J->new2old[p] * ldo + k] = x;
+    out[(int64_t)J->new2old[p] * s_ldo[k]] = x;
   }
 }
 
@@ -989,7 +1092,6 @@ struct WaveBuffers {
   const StepJob* jobs;
   const StepItem* items;
   LongChunk* chunks;
-  float* chunk_sum;
   int32_t* counters;  // [0] chunks of the wave, [1] jobs with running columns
 };
 
@@ -998,7 +1100,7 @@ static void run_wave(const Wave& wv, const WaveBuffers& B, int32_t max_iters, bo
   const StepItem* items = B.items + wv.item0;
   uint32_t* live_dev = (uint32_t*)B.counters + 1;
   GPR_CUDA(cudaMemsetAsync(B.counters, 0, 8, s));
-  ppr_start_kernel<T, W><<<wv.items, kStThreads, 0, s>>>(B.jobs, items, wv.per, B.chunks, B.counters, live_dev);
+  ppr_start_kernel<T, W><<<wv.items, kStThreads, 0, s>>>(B.jobs, items, B.chunks, B.counters, live_dev);
   GPR_CUDA(cudaGetLastError());
   int64_t launches = 2;
   const int long_grid = (int)std::min<int64_t>((wv.chunks + kStWarps - 1) / kStWarps, (int64_t)num_sms() * 8);
@@ -1010,13 +1112,13 @@ static void run_wave(const Wave& wv, const WaveBuffers& B, int32_t max_iters, bo
       if (live == 0) break;
     }
     if (long_grid > 0) {
-      ppr_long_kernel<T, W><<<long_grid, kStThreads, 0, s>>>(B.jobs, B.chunks, B.counters, it & 1, B.chunk_sum);
+      ppr_long_kernel<T, W><<<long_grid, kStThreads, 0, s>>>(B.jobs, B.chunks, B.counters, it);
       ++launches;
     }
-    ppr_rows_kernel<T, W><<<wv.items, kStThreads, 0, s>>>(B.jobs, items, wv.per, it & 1, B.chunk_sum, live_dev);
+    ppr_rows_kernel<T, W, false><<<wv.items, kStThreads, 0, s>>>(B.jobs, items, it, live_dev);
     ++launches;
   }
-  ppr_out_kernel<T, W><<<wv.items, kStThreads, 0, s>>>(B.jobs, items, wv.per);
+  ppr_out_kernel<T, W><<<wv.items, kStThreads, 0, s>>>(B.jobs, items);
   GPR_CUDA(cudaGetLastError());
   count_launches(launches);
 }
@@ -1074,10 +1176,9 @@ static void run_waves(const std::vector<StepRequest>& reqs, int32_t max_iters, b
       J.new2old = g->plan.new2old;
       J.n = g->n;
       J.m = g->m;
-      J.k = reqs[r].k;
       J.cols = reqs[r].cols;
-      J.max_iters = max_iters;
-      J.npieces = (int32_t)std::max<int64_t>(1, std::min<int64_t>((work(r) + kPieceWork - 1) / kPieceWork, g->n));
+      J.long_deg = kLongDeg;
+      J.npieces = ppr_pieces(g);
       // the job's part of the wave's workspace, as offsets for now
       auto take = [&](int64_t bytes) {
         const int64_t at = used;
@@ -1107,6 +1208,7 @@ static void run_waves(const std::vector<StepRequest>& reqs, int32_t max_iters, b
       wv.per = (int)std::max<int64_t>(1, std::min<int64_t>(kMaxPer, wv.work / (blocks * kStWarps * kPieceWork)));
       wv.item0 = (int32_t)items.size();
       for (int32_t j = wv.job0; j < wv.job0 + wv.jobs; ++j) {
+        jobs[j].per = wv.per;
         jobs[j].nitems = (jobs[j].npieces + kStWarps * wv.per - 1) / (kStWarps * wv.per);
         for (int32_t q = 0; q < jobs[j].nitems; ++q) items.push_back(StepItem{j, q});
       }
@@ -1132,7 +1234,8 @@ static void run_waves(const std::vector<StepRequest>& reqs, int32_t max_iters, b
     B.jobs = jobs_dev;
     B.items = items_dev;
     B.chunks = (LongChunk*)alloc((size_t)std::max<int64_t>(chunk_cap, 1) * sizeof(LongChunk));
-    B.chunk_sum = (float*)alloc((size_t)std::max<int64_t>(chunk_cells, 1) * 4);
+    float* chunk_sum = (float*)alloc((size_t)std::max<int64_t>(chunk_cells, 1) * 4);
+    for (StepJob& J : jobs) J.chunk_sum = chunk_sum;  // a wave's list is shared by its jobs
     B.counters = (int32_t*)alloc(8);
     *launched = true;
     GPR_CUDA(cudaMemcpyAsync(jobs_dev, jobs.data(), jobs.size() * sizeof(StepJob), cudaMemcpyHostToDevice, s));
@@ -1170,6 +1273,63 @@ void run_ppr_steps(const std::vector<StepRequest>& reqs, int32_t max_iters, bool
       if (launched || f.st != GPR_ENOMEM || wave_bytes / 8 < kMinWaveBytes) throw;
     }
   }
+}
+
+// ---- the server's slots ---------------------------------------------------------
+
+int32_t ppr_pieces(const gpr_graph* g) {
+  const int64_t work = g->m + 3 * (int64_t)g->n;
+  return (int32_t)std::max<int64_t>(1, std::min<int64_t>((work + kPieceWork - 1) / kPieceWork, g->n));
+}
+
+void ppr_piece_bounds(const gpr_graph* g, int32_t* prows, cudaStream_t s) {
+  const int32_t cnt = ppr_pieces(g);
+  ppr_graph_bounds_kernel<<<std::min(1024, cnt / 256 + 1), 256, 0, s>>>(g->col_ptr, g->n, g->m, cnt, prows);
+  GPR_CUDA(cudaGetLastError());
+  count_launches(1);
+}
+
+void heavy_of(const gpr_graph* g, const int32_t** rows, int32_t* n, int32_t* deg, int32_t* split0) {
+  const Plan& P = g->plan;
+  *rows = P.rows;
+  *n = 0;
+  *deg = INT_MAX;
+  *split0 = 0;
+  // the long rows are the last chunked (lanes 0) bucket; the plan's split
+  // entries list the rows of every chunked bucket in bucket order
+  int32_t before = 0;
+  for (int b = 0; b < P.nbuckets; ++b)
+    if (P.bucket[b].lanes == 0) {
+      *split0 = before;
+      *rows = P.rows + P.bucket[b].row_begin;
+      *n = P.bucket[b].row_end - P.bucket[b].row_begin;
+      *deg = b > 0 ? P.deg_threshold[b - 1] : -1;  // bucket 0 holds every degree from 0
+      before += *n;
+    }
+}
+
+template <typename T>
+static void slot_steps(const StepJob* jobs, const StepItem* items, int nitems, const StepItem* citems, int ncitems,
+                       int32_t steps, uint32_t* scratch, cudaStream_t s) {
+  ppr_join_kernel<T><<<nitems, kStThreads, 0, s>>>(jobs, items);
+  for (int32_t it = 0; it < steps; ++it) {
+    if (ncitems > 0) ppr_slot_long_kernel<T><<<ncitems, kStThreads, 0, s>>>(jobs, citems, it);
+    ppr_rows_kernel<T, kPprCols, true><<<nitems, kStThreads, 0, s>>>(jobs, items, it, scratch);
+  }
+  ppr_out_kernel<T, kPprCols><<<nitems, kStThreads, 0, s>>>(jobs, items);
+  GPR_CUDA(cudaGetLastError());
+  count_launches(2 + (int64_t)steps * (ncitems > 0 ? 2 : 1));
+}
+
+void ppr_slot_steps(const StepJob* jobs, const StepItem* items, int nitems, const StepItem* citems, int ncitems,
+                    int32_t steps, gpr_dtype dt, uint32_t* scratch, cudaStream_t s) {
+  if (nitems <= 0) return;
+  if (dt == GPR_BF16)
+    slot_steps<__nv_bfloat16>(jobs, items, nitems, citems, ncitems, steps, scratch, s);
+  else if (dt == GPR_FP16)
+    slot_steps<__half>(jobs, items, nitems, citems, ncitems, steps, scratch, s);
+  else
+    slot_steps<float>(jobs, items, nitems, citems, ncitems, steps, scratch, s);
 }
 
 }  // namespace gpr

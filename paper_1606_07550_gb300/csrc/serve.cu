@@ -10,12 +10,12 @@
 //      device budget allows; otherwise it waits.  While the head waits (at
 //      most kOvertakeMs), later requests may take free places of running
 //      slots, which needs no new slot;
-//   2. run steps_per_tick steps of every slot with live columns: each slot's
-//      rows are split into parts of about edges_per_part units of work (an
-//      edge counts 1, a row 3); per step, one launch gathers the long rows'
-//      edge chunks of every slot and one runs every (slot, part) (ppr.cu,
-//      ppr_step_kernel: new columns start at e_seed, finished ones freeze
-//      and are written to their result buffer by node id);
+//   2. run steps_per_tick steps of every slot with live columns on the
+//      step-major kernels (ppr_steps.cu): per step, one launch sums the long
+//      rows' edge chunks of every slot and one runs every item of every slot,
+//      each about edges_per_part units of work (an edge counts 1, a row 3); new
+//      columns start at e_seed, finished ones freeze and are written to their
+//      result buffer by node id after the last step;
 //   3. read back the column records, complete requests whose columns are
 //      all finished, free their places and slots that became empty.
 // A column's arithmetic does not depend on the other columns, so a result
@@ -44,17 +44,15 @@ constexpr int kOvertakeScan = 4096;
 struct Slot {
   int graph = -1;
   gpr_dtype dt = GPR_FP32;
-  float* X = nullptr;
-  void* C0 = nullptr;
+  float* X = nullptr;            // with BF16 deltas the running sums
+  void* C0 = nullptr;            // contributions, a row of zeros after the last
   void* C1 = nullptr;
-  float4* YS = nullptr;  // BF16 deltas: running and sent sums
+  float* S = nullptr;            // BF16 deltas: sent sums
   int32_t parity = 0;
   int64_t bytes = 0;
-  int32_t nparts = 1;
-  int32_t* part_rows = nullptr;  // device, nparts + 1
   PprCol* d_rec = nullptr;       // device, 64
-  ColState* d_st = nullptr;      // device, 2 x 64
-  double* d_psum = nullptr;      // device, 2 x nparts x 3 x 64
+  StepState* d_st = nullptr;     // device
+  int32_t* prows = nullptr;      // device, pieces + 1 row boundaries
   float* chunk_sum = nullptr;    // device, nchunks x 64: long-row chunk sums of a step
   PprCol cols[kPprCols];         // host mirror of d_rec
   uint64_t owner[kPprCols];      // ticket holding each place (0: free)
@@ -101,9 +99,10 @@ struct gpr_server {
   int alloc_attempts = 0;
   gpr_server_stats st{};
   // device staging for one tick
-  gpr::SlotDesc* d_desc = nullptr;
+  gpr::StepJob* d_desc = nullptr;
   gpr::StepItem* d_items = nullptr;
   gpr::StepItem* d_citems = nullptr;
+  uint32_t* d_scratch = nullptr;
   int cap_desc = 0, cap_items = 0, cap_citems = 0;
 };
 
@@ -111,31 +110,41 @@ namespace gpr {
 
 static size_t elem_bytes(gpr_dtype dt) { return dt == GPR_FP32 ? 4 : 2; }
 
-static int32_t parts_for(const gpr_server* S, const gpr_graph* g) {
-  // parts of about edges_per_part units of work (an edge; a row counts as 3)
+// Work of an item of g (an edge counts 1, a row 3): as configured, or for a
+// graph that fills the GPU with them small items, which end together, for a
+// smaller one twice as large ones, which leave the SMs to other slots.  A burst
+// of 32 requests over graphs of scales 14 to 22 takes 201 ms with items of 2^14
+// throughout, 229 with 2^15, 300 with 2^16 and 433 with 2^17.
+constexpr int64_t kLargeWork = 1 << 22;
+static int per_warp(const gpr_server* S, const gpr_graph* g) {
   const int64_t work = g->m + 3 * (int64_t)g->n;
-  const int64_t p = (work + S->cfg.edges_per_part - 1) / std::max<int64_t>(S->cfg.edges_per_part, 1);
-  return (int32_t)std::max<int64_t>(1, std::min<int64_t>(std::min<int64_t>(p, 1024), std::max(g->n, 1)));
+  const int64_t item = S->cfg.edges_per_part > 0 ? S->cfg.edges_per_part : work >= kLargeWork ? 1 << 14 : 1 << 15;
+  return (int)std::max<int64_t>(1, std::min<int64_t>(item / (kStWarps * kPieceWork), 1 << 20));
 }
 
-static int64_t slot_bytes(const gpr_server* S, const gpr_graph* g, gpr_dtype dt) {
-  const int64_t P = parts_for(S, g);
+static int64_t slot_bytes(const gpr_graph* g, gpr_dtype dt) {
   // per row and column: x and two contribution buffers, or with BF16 deltas
   // two delta buffers and the running and sent sums
-  return (int64_t)g->n * kPprCols * (dt == GPR_BF16 ? 2 * 2 + 8 : 4 + 2 * (int64_t)elem_bytes(dt)) + (P + 1) * 4 +
-         kPprCols * (int64_t)(sizeof(PprCol) + 2 * sizeof(ColState)) + 2 * P * 3 * kPprCols * 8 +
+  return (int64_t)g->n * kPprCols * (dt == GPR_BF16 ? 2 * 2 + 8 : 4 + 2 * (int64_t)elem_bytes(dt)) +
+         2 * kPprCols * (int64_t)elem_bytes(dt) + ((int64_t)ppr_pieces(g) + 1) * 4 +
+         kPprCols * (int64_t)sizeof(PprCol) + (int64_t)sizeof(StepState) +
          (int64_t)std::max(g->plan.nchunks, 1) * kPprCols * 4;
 }
 
-static void fill_desc(SlotDesc& D, const gpr_graph* g, const Slot* sl) {
-  D = SlotDesc{};
+static void fill_desc(StepJob& D, const gpr_server* S, const Slot* sl) {
+  const gpr_graph* g = S->pool[sl->graph];
+  D = StepJob{};
   D.col_ptr = g->col_ptr;
   D.row_idx = g->row_idx;
   D.inv_deg = g->plan.inv_deg;
   D.old2new = g->plan.old2new;
   D.new2old = g->plan.new2old;
+  D.m = g->m;
   D.n = g->n;
-  heavy_of(g, &D.heavy_rows, &D.n_heavy, &D.heavy_deg, &D.heavy_split0);
+  D.npieces = ppr_pieces(g);
+  D.per = per_warp(S, g);
+  D.nitems = (D.npieces + kStWarps * D.per - 1) / (kStWarps * D.per);
+  heavy_of(g, &D.heavy_rows, &D.n_heavy, &D.long_deg, &D.split0);
   D.chunk_begin = g->plan.chunk_begin;
   D.chunk_end = g->plan.chunk_end;
   D.split_hbeg = g->plan.split_hbeg;
@@ -143,31 +152,30 @@ static void fill_desc(SlotDesc& D, const gpr_graph* g, const Slot* sl) {
   D.split_cbeg = g->plan.split_cbeg;
   D.split_cend = g->plan.split_cend;
   D.nchunks = g->plan.nchunks;
-  D.chunk_sum = sl->chunk_sum;
-  D.nparts = sl->nparts;
-  D.part_rows = sl->part_rows;
+  D.prows = sl->prows;
   D.X = sl->X;
   D.C[0] = sl->C0;
   D.C[1] = sl->C1;
-  D.YS = sl->YS;
+  D.S = sl->S;
+  D.chunk_sum = sl->chunk_sum;
   D.parity = sl->parity;
-  D.rec = sl->d_rec;
-  D.st[0] = sl->d_st;
-  D.st[1] = sl->d_st + kPprCols;
-  D.psum[0] = sl->d_psum;
-  D.psum[1] = sl->d_psum + (int64_t)sl->nparts * 3 * kPprCols;
+  D.st = sl->d_st;
+  D.cols = sl->d_rec;
 }
 
-static void free_slot(gpr_server* S, Slot* sl) {
+static void free_slot_memory(gpr_server* S, Slot* sl) {
   dfree(sl->X, S->stream);
   dfree(sl->C0, S->stream);
   dfree(sl->C1, S->stream);
-  dfree(sl->YS, S->stream);
-  dfree(sl->part_rows, S->stream);
+  dfree(sl->S, S->stream);
   dfree(sl->d_rec, S->stream);
   dfree(sl->d_st, S->stream);
-  dfree(sl->d_psum, S->stream);
   dfree(sl->chunk_sum, S->stream);
+  dfree(sl->prows, S->stream);
+}
+
+static void free_slot(gpr_server* S, Slot* sl) {
+  free_slot_memory(S, sl);
   S->bytes_in_use -= sl->bytes;
   delete sl;
 }
@@ -184,7 +192,7 @@ static bool try_admit(gpr_server* S, Req& r, bool existing_only = false) {
       break;
     }
   if (existing_only && !target) return false;
-  const int64_t need = (target ? 0 : slot_bytes(S, g, r.dt)) + (int64_t)g->n * k * 4;
+  const int64_t need = (target ? 0 : slot_bytes(g, r.dt)) + (int64_t)g->n * k * 4;
   if (S->bytes_in_use + need > S->cfg.budget_bytes) return false;
   try {
     if (!target) {
@@ -194,29 +202,23 @@ static bool try_admit(gpr_server* S, Req& r, bool existing_only = false) {
       Slot* sl = new Slot();
       sl->graph = r.graph;
       sl->dt = r.dt;
-      sl->bytes = slot_bytes(S, g, r.dt);
-      sl->nparts = parts_for(S, g);
+      sl->bytes = slot_bytes(g, r.dt);
       try {
-        if (r.dt != GPR_BF16) sl->X = (float*)dalloc((size_t)g->n * kPprCols * 4, S->stream);
-        sl->C0 = dalloc((size_t)g->n * kPprCols * elem_bytes(r.dt), S->stream);
-        sl->C1 = dalloc((size_t)g->n * kPprCols * elem_bytes(r.dt), S->stream);
-        if (r.dt == GPR_BF16) sl->YS = (float4*)dalloc((size_t)g->n * kPprCols * 8, S->stream);
-        sl->part_rows = (int32_t*)dalloc(((size_t)sl->nparts + 1) * 4, S->stream);
+        const size_t cells = (size_t)g->n * kPprCols, tsz = elem_bytes(r.dt);
+        sl->X = (float*)dalloc(cells * 4, S->stream);
+        sl->C0 = dalloc((cells + kPprCols) * tsz, S->stream);
+        sl->C1 = dalloc((cells + kPprCols) * tsz, S->stream);
+        if (r.dt == GPR_BF16) sl->S = (float*)dalloc(cells * 4, S->stream);
         sl->d_rec = (PprCol*)dalloc(kPprCols * sizeof(PprCol), S->stream);
-        sl->d_st = (ColState*)dalloc(2 * kPprCols * sizeof(ColState), S->stream);
-        sl->d_psum = (double*)dalloc((size_t)2 * sl->nparts * 3 * kPprCols * 8, S->stream);
+        sl->d_st = (StepState*)dalloc(sizeof(StepState), S->stream);
         sl->chunk_sum = (float*)dalloc((size_t)std::max(g->plan.nchunks, 1) * kPprCols * 4, S->stream);
-        ppr_part_bounds(g->col_ptr, g->n, g->m, sl->nparts, sl->part_rows, S->stream);
+        sl->prows = (int32_t*)dalloc(((size_t)ppr_pieces(g) + 1) * 4, S->stream);
+        ppr_piece_bounds(g, sl->prows, S->stream);
+        GPR_CUDA(cudaMemsetAsync((char*)sl->C0 + cells * tsz, 0, kPprCols * tsz, S->stream));
+        GPR_CUDA(cudaMemsetAsync((char*)sl->C1 + cells * tsz, 0, kPprCols * tsz, S->stream));
+        GPR_CUDA(cudaMemsetAsync(sl->d_st, 0, sizeof(StepState), S->stream));
       } catch (...) {
-        dfree(sl->X, S->stream);
-        dfree(sl->C0, S->stream);
-        dfree(sl->C1, S->stream);
-        dfree(sl->YS, S->stream);
-        dfree(sl->part_rows, S->stream);
-        dfree(sl->d_rec, S->stream);
-        dfree(sl->d_st, S->stream);
-        dfree(sl->d_psum, S->stream);
-        dfree(sl->chunk_sum, S->stream);
+        free_slot_memory(S, sl);
         delete sl;
         throw;
       }
@@ -281,45 +283,40 @@ static V* grow(V* p, int& cap, int need, cudaStream_t s) {
   return (V*)dalloc((size_t)cap * sizeof(V), s);
 }
 
-// One tick: per storage type, kStepInit, steps_per_tick run launches and
-// kStepFinish over every (slot, part) of the slots with live columns, then
-// the records come back.  Runs without the lock: only the scheduler thread
-// touches slots.
+// One tick: per storage type, steps_per_tick steps of every item of the slots
+// with live columns, then the records come back.  Runs without the lock: only
+// the scheduler thread touches slots.
 static void run_tick(gpr_server* S, const std::vector<Slot*>& live) {
-  std::vector<SlotDesc> desc(live.size());
+  std::vector<StepJob> desc(live.size());
   for (size_t i = 0; i < live.size(); ++i) {
     Slot* sl = live[i];
-    fill_desc(desc[i], S->pool[sl->graph], sl);
+    fill_desc(desc[i], S, sl);
     GPR_CUDA(cudaMemcpyAsync(sl->d_rec, sl->cols, kPprCols * sizeof(PprCol), cudaMemcpyHostToDevice, S->stream));
   }
   S->d_desc = grow(S->d_desc, S->cap_desc, (int)desc.size(), S->stream);
-  GPR_CUDA(cudaMemcpyAsync(S->d_desc, desc.data(), desc.size() * sizeof(SlotDesc), cudaMemcpyHostToDevice, S->stream));
+  GPR_CUDA(cudaMemcpyAsync(S->d_desc, desc.data(), desc.size() * sizeof(StepJob), cudaMemcpyHostToDevice, S->stream));
   const int32_t T = S->cfg.steps_per_tick;
   for (gpr_dtype dt : {GPR_FP32, GPR_BF16, GPR_FP16}) {
-    std::vector<StepItem> items;
+    std::vector<StepItem> items, citems;  // citems: long-row chunks of the same slots
+    std::vector<size_t> order;            // the slots with the largest items first
     for (size_t i = 0; i < live.size(); ++i)
-      if (live[i]->dt == dt)
-        for (int32_t q = 0; q < live[i]->nparts; ++q) items.push_back(StepItem{(int32_t)i, q});
+      if (live[i]->dt == dt) order.push_back(i);
+    std::stable_sort(order.begin(), order.end(), [&](size_t a, size_t b) { return desc[a].per > desc[b].per; });
+    for (size_t i : order) {
+      for (int32_t q = 0; q < desc[i].nitems; ++q) items.push_back(StepItem{(int32_t)i, q});
+      for (int32_t q = 0; q * kStWarps < desc[i].nchunks; ++q) citems.push_back(StepItem{(int32_t)i, q});
+    }
     if (items.empty()) continue;
-    S->d_items = grow(S->d_items, S->cap_items, (int)items.size(), S->stream);
+    const int32_t ni = (int32_t)items.size(), nci = (int32_t)citems.size();
+    S->d_items = grow(S->d_items, S->cap_items, ni, S->stream);
     GPR_CUDA(cudaMemcpyAsync(S->d_items, items.data(), items.size() * sizeof(StepItem), cudaMemcpyHostToDevice,
                              S->stream));
-    std::vector<StepItem> citems;  // long-row chunk groups of the same slots
-    for (size_t i = 0; i < live.size(); ++i)
-      if (live[i]->dt == dt)
-        for (int32_t q = 0; q * kChunksPerItem < desc[i].nchunks; ++q) citems.push_back(StepItem{(int32_t)i, q});
-    const int32_t ni = (int32_t)items.size(), nci = (int32_t)citems.size();
     if (nci > 0) {
       S->d_citems = grow(S->d_citems, S->cap_citems, nci, S->stream);
       GPR_CUDA(cudaMemcpyAsync(S->d_citems, citems.data(), citems.size() * sizeof(StepItem),
                                cudaMemcpyHostToDevice, S->stream));
     }
-    ppr_step_launch(S->d_desc, S->d_items, ni, kStepInit, 0, dt, S->stream);
-    for (int32_t st = 1; st <= T; ++st) {
-      ppr_chunk_launch(S->d_desc, S->d_citems, nci, st, dt, S->stream);
-      ppr_step_launch(S->d_desc, S->d_items, ni, kStepRun, st, dt, S->stream);
-    }
-    ppr_step_launch(S->d_desc, S->d_items, ni, kStepFinish, T + 1, dt, S->stream);
+    ppr_slot_steps(S->d_desc, S->d_items, ni, S->d_citems, nci, T, dt, S->d_scratch, S->stream);
     // the host copy of `items` must outlive the copy above
     GPR_CUDA(cudaStreamSynchronize(S->stream));
   }
@@ -472,7 +469,6 @@ gpr_status serve_create(const gpr_graph* const* pool, int32_t num_graphs, const 
   S->cfg = *cfg;
   if (S->cfg.max_queue <= 0) S->cfg.max_queue = 65536;
   if (S->cfg.steps_per_tick <= 0) S->cfg.steps_per_tick = 8;
-  if (S->cfg.edges_per_part <= 0) S->cfg.edges_per_part = (int64_t)1 << 18;
   std::vector<const gpr_graph*> uniq(S->pool);
   std::sort(uniq.begin(), uniq.end());
   uniq.erase(std::unique(uniq.begin(), uniq.end()), uniq.end());
@@ -485,13 +481,16 @@ gpr_status serve_create(const gpr_graph* const* pool, int32_t num_graphs, const 
   }
   try {
     GPR_CUDA(cudaStreamCreateWithFlags(&S->stream, cudaStreamNonBlocking));
+    S->d_scratch = (uint32_t*)dalloc(4, S->stream);
   } catch (const StatusFail& f) {
+    dfree(S->d_scratch, S->stream);
     if (S->stream) cudaStreamDestroy(S->stream);
     delete S;
     set_error("serve_create: %s", f.msg.c_str());
     return f.st;
   } catch (const CudaFail& f) {
     cudaGetLastError();
+    dfree(S->d_scratch, S->stream);
     if (S->stream) cudaStreamDestroy(S->stream);
     delete S;
     set_error("serve_create: %s failed: %s", f.what, cudaGetErrorString(f.err));
@@ -527,7 +526,7 @@ gpr_status serve_submit(gpr_server* S, const gpr_request* r, uint64_t* ticket) {
     set_error("serve_submit: damping, tol, max_iters or dtype out of range");
     return GPR_EINVAL;
   }
-  const int64_t alone = S->pool_bytes + slot_bytes(S, g, r->dt) + (int64_t)g->n * r->num_seeds * 4;
+  const int64_t alone = S->pool_bytes + slot_bytes(g, r->dt) + (int64_t)g->n * r->num_seeds * 4;
   std::lock_guard<std::mutex> lk(S->mu);
   ++S->st.submitted;
   if (alone > S->cfg.budget_bytes) {
@@ -691,6 +690,7 @@ gpr_status serve_destroy(gpr_server* S) {
   dfree(S->d_desc, S->stream);
   dfree(S->d_items, S->stream);
   dfree(S->d_citems, S->stream);
+  dfree(S->d_scratch, S->stream);
   cudaError_t e = cudaStreamSynchronize(S->stream);
   cudaStreamDestroy(S->stream);
   delete S;
