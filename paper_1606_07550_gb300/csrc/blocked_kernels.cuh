@@ -382,7 +382,8 @@ __global__ void __launch_bounds__(kBkThreads, 1) bk_accum_kernel(
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, nwarps = blockDim.x >> 5;
   // this warp's two staging slots: 256 codes or packed words, then 256 row ids
   unsigned char* w_stage = reinterpret_cast<unsigned char*>(s_acc32 + 2 * W) + (size_t)warp * 2 * kAccumSlotBytes;
-  // thread 0 fetches the next unit while the current one is added
+  // thread 0 fetches the next unit while the current one's rows are finished
+  // (earlier would hold a unit that an idle block could take)
   auto fetch = [&](int at) {
     const int32_t u = (int32_t)(atomicAdd(ctr + 1, 1u) - epoch);
     const bool ok = u >= 0 && u < nunits;
@@ -403,7 +404,6 @@ __global__ void __launch_bounds__(kBkThreads, 1) bk_accum_kernel(
       for (int32_t i = tid; i < nq; i += blockDim.x) z_lo[i] = z_hi[i] = make_uint4(0u, 0u, 0u, 0u);
     }
     __syncthreads();
-    if (tid == 0) fetch(at ^ 1);
     // Lane l handles edges 4l..4l+3 and 128+4l..128+4l+3 of each 256-edge
     // chunk; it copies exactly those words (and row ids) into its slot while
     // the previous chunk is added.  An edge outside the unit's range (in a
@@ -531,6 +531,7 @@ __global__ void __launch_bounds__(kBkThreads, 1) bk_accum_kernel(
       cp_async_wait<0>();
     }
     __syncthreads();
+    if (tid == 0) fetch(at ^ 1);
     if (un.nparts > 1) {
       unsigned long long* g = acc_g + (int64_t)un.split * W;
       for (int32_t i = tid; i < nv; i += blockDim.x) {
