@@ -239,30 +239,50 @@ __global__ void digit_starts_kernel(const uint32_t* __restrict__ hist, DigitPlan
 // warp-striped (item j of warp w is tile position w*512 + j*32 + lane), so
 // (warp, item, lane) order is input order and the per-warp match-based
 // ranking keeps the sort stable.  Thread t owns digits kDPT*t .. kDPT*t +
-// kDPT - 1 for the tile's scans and look-backs.
+// kDPT - 1 for the tile's scans and look-backs (the first kRadix / kDPT
+// threads own them all).
 // kBatch: predecessors read per look-back round trip; a sort of few tiles, all
 // resident at once and each waiting on the others' counts, takes more.
-template <int kBits, int kShift, int kBatch = 4>
-__global__ void __launch_bounds__(kThreads, 4) onesweep_kernel(
+//
+// What bounds it.  DRAM is at 35%: a key costs ranking.  By votes alone (one a
+// digit bit) the ALU pipe is the limit (68% busy, 153 instructions per 32
+// keys; 444 us a pass over 69 M keys); by masks in shared memory alone, where
+// the lanes of a digit meet by atomic or, the shared-memory pipe (83%, 447 us).
+// Half of the items each way: 400 us.  512 threads a tile instead of 256
+// halve the look-backs and double the runs that a digit writes (9-bit digits
+// of 4.8 M keys: 83 -> 37 us with both).
+template <int kT, int kBits>
+struct SweepShared {
+  uint64_t keys[kT * kItems];
+  uint32_t wcnt[kT / 32][1 << kBits];
+  uint64_t goff[1 << kBits];
+  uint32_t wsum[kT / 32];
+  uint32_t tile;
+};
+template <int kT, int kBits, int kShift, int kBatch = 4>
+__global__ void __launch_bounds__(kT, 1024 / kT) onesweep_kernel(
     const uint64_t* __restrict__ in, uint64_t* __restrict__ out, int64_t n, int shift_arg,
     const uint32_t* __restrict__ dstart, uint64_t* __restrict__ status, uint32_t* __restrict__ tile_ctr,
     uint32_t epoch, int* __restrict__ derr) {
   const int shift = kShift >= 0 ? kShift : shift_arg;
   constexpr int kRadix = 1 << kBits;
   constexpr uint32_t kMask = kRadix - 1;
-  constexpr int kDPT = kRadix / kThreads;
-  static_assert(kDPT >= 1 && kDPT * kThreads == kRadix, "whole digits per thread");
-  __shared__ uint64_t s_keys[kTile];
-  __shared__ uint32_t s_wcnt[kWarps][kRadix];
-  __shared__ uint64_t s_goff[kRadix];
-  __shared__ uint32_t s_wsum[kWarps];
-  __shared__ uint32_t s_tile;
+  constexpr int kTileKeys = kT * kItems, kNW = kT / 32;
+  constexpr int kDPT = kRadix > kT ? kRadix / kT : 1;
+  static_assert(kRadix % 32 == 0 && kDPT * kT % kRadix == 0, "whole digits per thread, whole warps of them");
+  extern __shared__ __align__(16) unsigned char sweep_shared[];
+  SweepShared<kT, kBits>& sh = *reinterpret_cast<SweepShared<kT, kBits>*>(sweep_shared);
+  auto& s_keys = sh.keys;
+  auto& s_wcnt = sh.wcnt;
+  auto& s_goff = sh.goff;
+  auto& s_wsum = sh.wsum;
   const int t = threadIdx.x, w = t >> 5, lane = t & 31;
-  if (t == 0) s_tile = atomicAdd(tile_ctr, 1u);
-  for (int i = t; i < kWarps * kRadix; i += kThreads) (&s_wcnt[0][0])[i] = 0;
+  if (t == 0) sh.tile = atomicAdd(tile_ctr, 1u);
+  for (int i = t; i < kNW * kRadix; i += kT) (&s_wcnt[0][0])[i] = 0;
+  for (int i = t; i < kTileKeys / 2; i += kT) reinterpret_cast<uint4*>(s_keys)[i] = make_uint4(0, 0, 0, 0);
   __syncthreads();
-  const int64_t tile = s_tile;
-  const int64_t base = tile * kTile + (int64_t)w * (kItems * 32) + lane;
+  const int64_t tile = sh.tile;
+  const int64_t base = tile * kTileKeys + (int64_t)w * (kItems * 32) + lane;
 
   uint64_t k[kItems];
 #pragma unroll
@@ -272,66 +292,91 @@ __global__ void __launch_bounds__(kThreads, 4) onesweep_kernel(
   }
   uint32_t rk[kItems / 2] = {};  // ranks in the warp (< 512), two 16-bit halves per word
   const uint32_t lt = lanemask_lt();
+  constexpr int kGroup = kTileKeys * 2 / (kNW * kRadix);  // items whose masks fit the warp's part of s_keys
+  constexpr int kMasked = kGroup / 2;                        // of them, by masks
+  static_assert(kGroup >= 2 && kItems % kGroup == 0, "whole groups of items");
+  uint32_t* masks = reinterpret_cast<uint32_t*>(s_keys) + w * (kGroup * kRadix);
 #pragma unroll
-  for (int j = 0; j < kItems; ++j) {
-    const uint32_t d = (uint32_t)(k[j] >> shift) & kMask;
-    // the lanes holding the same digit: one vote per digit bit
-    uint32_t peers = 0xffffffffu;
+  for (int j0 = 0; j0 < kItems; j0 += kGroup) {
+    uint32_t peers[kGroup];
 #pragma unroll
-    for (int bb = 0; bb < kBits; ++bb) {
-      const uint32_t bit = (d >> bb) & 1u;
-      const uint32_t vote = __ballot_sync(0xffffffffu, bit);
-      peers &= bit ? vote : ~vote;
+    for (int j = 0; j < kMasked; ++j)
+      atomicOr(&masks[j * kRadix + ((uint32_t)(k[j0 + j] >> shift) & kMask)], 1u << lane);
+#pragma unroll
+    for (int j = kMasked; j < kGroup; ++j) {
+      const uint32_t d = (uint32_t)(k[j0 + j] >> shift) & kMask;
+      peers[j] = 0xffffffffu;
+#pragma unroll
+      for (int bb = 0; bb < kBits; ++bb) {
+        const bool bit = (d >> bb) & 1u;
+        const uint32_t vote = __ballot_sync(0xffffffffu, bit);
+        peers[j] &= vote ^ (bit ? 0u : ~0u);
+      }
     }
-    const uint32_t c = s_wcnt[w][d];
-    rk[j >> 1] |= (c + __popc(peers & lt)) << (16 * (j & 1));
     __syncwarp();
-    if ((peers & lt) == 0) s_wcnt[w][d] = c + __popc(peers);
+#pragma unroll
+    for (int j = 0; j < kMasked; ++j) peers[j] = masks[j * kRadix + ((uint32_t)(k[j0 + j] >> shift) & kMask)];
     __syncwarp();
+#pragma unroll
+    for (int j = 0; j < kGroup; ++j) {
+      const uint32_t d = (uint32_t)(k[j0 + j] >> shift) & kMask;
+      const uint32_t c = s_wcnt[w][d];
+      const uint32_t before = __popc(peers[j] & lt);
+      rk[(j0 + j) >> 1] |= (c + before) << (16 * ((j0 + j) & 1));
+      __syncwarp();
+      if (before == 0) {
+        s_wcnt[w][d] = c + __popc(peers[j]);
+        if (j < kMasked) masks[j * kRadix + d] = 0;
+      }
+      __syncwarp();
+    }
   }
   __syncthreads();
 
   // per owned digit: per-warp exclusive offsets and the tile count
-  uint32_t cnt[kDPT];
-  uint32_t tsum = 0;
+  const bool owner = kDPT * t < kRadix;  // (whole warps)
+  uint32_t cnt[kDPT], tstart[kDPT];
+  uint32_t tsum = 0, v = 0;
+  if (owner) {
 #pragma unroll
-  for (int q = 0; q < kDPT; ++q) {
-    const int d = kDPT * t + q;
-    uint32_t c = 0;
+    for (int q = 0; q < kDPT; ++q) {
+      const int d = kDPT * t + q;
+      uint32_t c = 0;
 #pragma unroll
-    for (int ww = 0; ww < kWarps; ++ww) {
-      const uint32_t v = s_wcnt[ww][d];
-      s_wcnt[ww][d] = c;
-      c += v;
+      for (int ww = 0; ww < kNW; ++ww) {
+        const uint32_t x = s_wcnt[ww][d];
+        s_wcnt[ww][d] = c;
+        c += x;
+      }
+      cnt[q] = c;
+      tsum += c;
+      if (tile == 0)
+        st_relaxed_u64(status + d, lb_word(epoch, kFlagInc, c));
+      else
+        st_relaxed_u64(status + tile * kRadix + d, lb_word(epoch, kFlagAgg, c));
     }
-    cnt[q] = c;
-    tsum += c;
-    if (tile == 0)
-      st_relaxed_u64(status + d, lb_word(epoch, kFlagInc, c));
-    else
-      st_relaxed_u64(status + tile * kRadix + d, lb_word(epoch, kFlagAgg, c));
-  }
-
-  // tile-local exclusive scan over digits (thread order is digit order)
-  uint32_t v = tsum;
+    // tile-local exclusive scan over digits (thread order is digit order)
+    v = tsum;
 #pragma unroll
-  for (int o = 1; o < 32; o <<= 1) {
-    uint32_t y = __shfl_up_sync(0xffffffffu, v, o);
-    if (lane >= o) v += y;
+    for (int o = 1; o < 32; o <<= 1) {
+      uint32_t y = __shfl_up_sync(0xffffffffu, v, o);
+      if (lane >= o) v += y;
+    }
+    if (lane == 31) s_wsum[w] = v;
   }
-  if (lane == 31) s_wsum[w] = v;
   __syncthreads();
-  uint32_t woff = 0;
-  for (int ww = 0; ww < w; ++ww) woff += s_wsum[ww];
-  uint32_t tstart[kDPT];
-  tstart[0] = woff + v - tsum;
+  if (owner) {
+    uint32_t woff = 0;
+    for (int ww = 0; ww < w; ++ww) woff += s_wsum[ww];
+    tstart[0] = woff + v - tsum;
 #pragma unroll
-  for (int q = 1; q < kDPT; ++q) tstart[q] = tstart[q - 1] + cnt[q - 1];
-  // s_wcnt[w][d]: where warp w's first key of digit d goes in the tile
+    for (int q = 1; q < kDPT; ++q) tstart[q] = tstart[q - 1] + cnt[q - 1];
+    // s_wcnt[w][d]: where warp w's first key of digit d goes in the tile
 #pragma unroll
-  for (int q = 0; q < kDPT; ++q)
+    for (int q = 0; q < kDPT; ++q)
 #pragma unroll
-    for (int ww = 0; ww < kWarps; ++ww) s_wcnt[ww][kDPT * t + q] += tstart[q];
+      for (int ww = 0; ww < kNW; ++ww) s_wcnt[ww][kDPT * t + q] += tstart[q];
+  }
   __syncthreads();
 
   // the tile in digit order in shared memory, before the look-back, so that
@@ -342,27 +387,29 @@ __global__ void __launch_bounds__(kThreads, 4) onesweep_kernel(
     s_keys[s_wcnt[w][d] + ((rk[j >> 1] >> (16 * (j & 1))) & 0xFFFFu)] = k[j];
   }
 
+  if (owner) {
 #pragma unroll
-  for (int q = 0; q < kDPT; ++q) {
-    const int d = kDPT * t + q;
-    uint64_t excl = 0;
-    if (tile != 0) {
-      excl = lookback<kBatch>(status + d, tile, kRadix, epoch, derr);
-      st_relaxed_u64(status + tile * kRadix + d, lb_word(epoch, kFlagInc, excl + cnt[q]));
+    for (int q = 0; q < kDPT; ++q) {
+      const int d = kDPT * t + q;
+      uint64_t excl = 0;
+      if (tile != 0) {
+        excl = lookback<kBatch>(status + d, tile, kRadix, epoch, derr);
+        st_relaxed_u64(status + tile * kRadix + d, lb_word(epoch, kFlagInc, excl + cnt[q]));
+      }
+      // output index of tile position i with digit d: s_goff[d] + i (the digit's
+      // global start is at least its tile-local start, so no wrap)
+      s_goff[d] = (uint64_t)dstart[d] + excl - tstart[q];
     }
-    // output index of tile position i with digit d: s_goff[d] + i (the digit's
-    // global start is at least its tile-local start, so no wrap)
-    s_goff[d] = (uint64_t)dstart[d] + excl - tstart[q];
   }
   __syncthreads();
-  if ((tile + 1) * kTile <= n) {  // a full tile: every index is below n
+  if ((tile + 1) * kTileKeys <= n) {  // a full tile: every index is below n
 #pragma unroll 4
-    for (int i = t; i < kTile; i += kThreads) {
+    for (int i = t; i < kTileKeys; i += kT) {
       const uint64_t key = s_keys[i];
       out[s_goff[(uint32_t)(key >> shift) & kMask] + (uint64_t)i] = key;
     }
   } else {
-    for (int i = t; i < kTile; i += kThreads) {
+    for (int i = t; i < kTileKeys; i += kT) {
       const uint64_t key = s_keys[i];
       const uint64_t dst = s_goff[(uint32_t)(key >> shift) & kMask] + (uint64_t)i;
       if (dst < (uint64_t)n) out[dst] = key;
@@ -372,23 +419,54 @@ __global__ void __launch_bounds__(kThreads, 4) onesweep_kernel(
 
 using SweepKernel = void (*)(const uint64_t*, uint64_t*, int64_t, int, const uint32_t*, uint64_t*, uint32_t*,
                             uint32_t, int*);
+constexpr int kManyThreads = 512;
+struct Sweep {
+  SweepKernel f;
+  int threads;
+  size_t shared;
+};
+template <int kT, int kBits, int kShift, int kBatch = 4>
+static Sweep sweep() {
+  return {onesweep_kernel<kT, kBits, kShift, kBatch>, kT, sizeof(SweepShared<kT, kBits>)};
+}
 // 8-bit passes at whole bytes (shift fixed at compile time), 9-bit passes
-static const SweepKernel kSweep8[8] = {onesweep_kernel<8, 0>,  onesweep_kernel<8, 8>,  onesweep_kernel<8, 16>,
-                                       onesweep_kernel<8, 24>, onesweep_kernel<8, 32>, onesweep_kernel<8, 40>,
-                                       onesweep_kernel<8, 48>, onesweep_kernel<8, 56>};
-static const SweepKernel kSweep8Any = onesweep_kernel<8, -1>;
-static const SweepKernel kSweep9 = onesweep_kernel<9, -1>;
-// sorts of up to kFewTiles tiles
-static const SweepKernel kSweep8Few = onesweep_kernel<8, -1, 16>;
-static const SweepKernel kSweep9Few = onesweep_kernel<9, -1, 16>;
+static const Sweep kSweep8[8] = {sweep<kManyThreads, 8, 0>(),  sweep<kManyThreads, 8, 8>(),  sweep<kManyThreads, 8, 16>(), sweep<kManyThreads, 8, 24>(),
+                                 sweep<kManyThreads, 8, 32>(), sweep<kManyThreads, 8, 40>(), sweep<kManyThreads, 8, 48>(), sweep<kManyThreads, 8, 56>()};
+static const Sweep kSweep8Any = sweep<kManyThreads, 8, -1>();
+static const Sweep kSweep9 = sweep<kManyThreads, 9, -1>();
+// Sorts of up to kFewTiles tiles of 4,096 keys: a tile an SM, where larger
+// tiles would leave SMs idle.  With the line at 608 tiles a build of 1.5 M edges
+// takes 371 us instead of 353 and one of 2 M 435 instead of 386.
+static const Sweep kSweep8Few = sweep<256, 8, -1, 16>();
+static const Sweep kSweep9Few = sweep<256, 9, -1, 16>();
 constexpr int64_t kFewTiles = 152;
+
+// The largest shared-memory carve-out and the blocks' shared memory, once a device.
+static void sweep_attributes() {
+  static std::once_flag done[64];
+  const int dev = device_ordinal();
+  auto set = [] {
+    auto one = [](const Sweep& w) {
+      GPR_CUDA(cudaFuncSetAttribute(w.f, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)w.shared));
+      GPR_CUDA(cudaFuncSetAttribute(w.f, cudaFuncAttributePreferredSharedMemoryCarveout,
+                                    (int)cudaSharedmemCarveoutMaxShared));
+    };
+    for (const Sweep& w : kSweep8) one(w);
+    for (const Sweep& w : {kSweep8Any, kSweep9, kSweep8Few, kSweep9Few}) one(w);
+  };
+  if (dev >= 0 && dev < 64)
+    std::call_once(done[dev], set);
+  else
+    set();
+}
 
 uint64_t* radix_sort_u64(uint64_t* keys, uint64_t* alt, int64_t n, int bits, cudaStream_t s,
                          int* derr, uint32_t* hist_in, int low) {
   const DigitPlan dp = digit_plan(bits, low);
   const int passes = dp.passes;
   if (n <= 1 || passes == 0) return keys;
-  const int64_t tiles = (n + kTile - 1) / kTile;
+  const bool few = n <= kFewTiles * kTile;
+  const int64_t tile_keys = (few ? 256 : kManyThreads) * kItems, tiles = (n + tile_keys - 1) / tile_keys;
   int radix = 0;
   for (int p = 0; p < passes; ++p) radix = std::max(radix, 1 << dp.width[p]);
   uint32_t* hist = hist_in;
@@ -414,24 +492,17 @@ uint64_t* radix_sort_u64(uint64_t* keys, uint64_t* alt, int64_t n, int bits, cud
     digit_starts_kernel<<<passes, kMaxRadix, 0, s>>>(hist, dp, starts);
     GPR_CUDA(cudaGetLastError());
     count_launches(1);
-    static std::once_flag carveout;  // four blocks per SM need the largest shared-memory carve-out
-    std::call_once(carveout, [] {
-      for (SweepKernel f : kSweep8)
-        cudaFuncSetAttribute(f, cudaFuncAttributePreferredSharedMemoryCarveout, (int)cudaSharedmemCarveoutMaxShared);
-      for (SweepKernel f : {kSweep8Any, kSweep9, kSweep8Few, kSweep9Few})
-        cudaFuncSetAttribute(f, cudaFuncAttributePreferredSharedMemoryCarveout, (int)cudaSharedmemCarveoutMaxShared);
-    });
+    sweep_attributes();
     uint64_t* a = keys;
     uint64_t* b = alt;
     for (int p = 0; p < passes; ++p) {
       // (8-bit digits of a whole sort start at whole bytes until the first 9-bit one)
-      const bool few = tiles <= kFewTiles;
-      const SweepKernel f = dp.width[p] == 9          ? (few ? kSweep9Few : kSweep9)
+      const Sweep& f = dp.width[p] == 9          ? (few ? kSweep9Few : kSweep9)
                             : few                     ? kSweep8Few
                             : (dp.shift[p] % 8) == 0 ? kSweep8[dp.shift[p] / 8]
                                                       : kSweep8Any;
-      f<<<(unsigned)tiles, kThreads, 0, s>>>(a, b, n, dp.shift[p], starts + kMaxRadix * p, status, ctr + p,
-                                             (uint32_t)(p + 1), derr);
+      f.f<<<(unsigned)tiles, f.threads, f.shared, s>>>(a, b, n, dp.shift[p], starts + kMaxRadix * p, status, ctr + p,
+                                                       (uint32_t)(p + 1), derr);
       GPR_CUDA(cudaGetLastError());
       count_launches(1);
       std::swap(a, b);
@@ -583,31 +654,14 @@ __device__ __forceinline__ void fill_rows(int32_t* col_ptr, int32_t first, int32
   }
 }
 
-// Neighbours of item j in input order, for warp-striped tiles.  All lanes
-// take part in the shuffles; only lane 0 / lane 31 at a warp's first / last
-// item read global memory.  kSentinel stands for "no neighbour".
-__device__ __forceinline__ uint64_t prev_key(const uint64_t (&k)[kItems], int j, int lane, int64_t i,
-                                             const uint64_t* __restrict__ keys, int64_t m_raw) {
-  const uint64_t up = __shfl_up_sync(0xffffffffu, k[j], 1);
-  const uint64_t row_last = __shfl_sync(0xffffffffu, k[j > 0 ? j - 1 : 0], 31);
-  if (lane > 0) return up;
-  if (j > 0) return row_last;
-  return (i > 0 && i - 1 < m_raw) ? keys[i - 1] : kSentinel;
-}
-__device__ __forceinline__ uint64_t next_key(const uint64_t (&k)[kItems], int j, int lane, int64_t i,
-                                             const uint64_t* __restrict__ keys, int64_t m_raw) {
-  const uint64_t down = __shfl_down_sync(0xffffffffu, k[j], 1);
-  const uint64_t row_first = __shfl_sync(0xffffffffu, k[j + 1 < kItems ? j + 1 : j], 0);
-  if (lane < 31) return down;
-  if (j + 1 < kItems) return row_first;
-  return i + 1 < m_raw ? keys[i + 1] : kSentinel;
-}
-
 // Sorted keys -> CSC.  Item j of warp w is tile position w*512 + j*32 + lane
 // (input order), so the ballot counts give each kept key its output index.
 // Keeps the first of each run of equal keys and drops sentinels; writes
 // row_idx, the row starts (gaps of empty rows filled) and out-degrees.
-__global__ void __launch_bounds__(kThreads) dedupe_kernel(
+// Bound by its instructions and by waiting at the barrier for the look-back:
+// a warp's look-back over 32 predecessors and half the shuffles took 69 M keys
+// from 473 to 417 us (the bytes alone are 122 us).
+__global__ void __launch_bounds__(kThreads, 4) dedupe_kernel(
     const uint64_t* __restrict__ keys, int64_t m_raw, int b, int32_t n, int32_t* __restrict__ row_idx,
     int32_t* __restrict__ col_ptr, int32_t* __restrict__ outdeg, uint64_t* __restrict__ status,
     uint32_t* __restrict__ tile_ctr, int64_t* __restrict__ m_out, Gap* __restrict__ gaps,
@@ -629,57 +683,67 @@ __global__ void __launch_bounds__(kThreads) dedupe_kernel(
     int64_t i = base + j * 32;
     k[j] = i < m_raw ? __ldcs(keys + i) : kSentinel;
   }
+  // Neighbours come by shuffle (warp-striped: the key before lane 0's is lane
+  // 31's of the item before), a key's once: for whether it is kept; a row's
+  // start and the last key need only the row and whether there is a key.
   uint32_t ballot[kItems];
-  uint32_t wtotal = 0;
+  uint32_t wtotal = 0, nvalid = 0;  // kept keys, and keys at all (which come first), of the warp
+  uint64_t before = kSentinel;  // the key before the warp's first
+  if (base - lane > 0 && base - lane <= m_raw) before = keys[base - lane - 1];
+  uint64_t last = before;
 #pragma unroll
   for (int j = 0; j < kItems; ++j) {
-    const int64_t i = base + j * 32;
-    const uint64_t prev = prev_key(k, j, lane, i, keys, m_raw);
-    const bool keep = (k[j] != kSentinel) && (i == 0 || k[j] != prev);
-    ballot[j] = __ballot_sync(0xffffffffu, keep);
+    uint64_t prev = __shfl_up_sync(0xffffffffu, k[j], 1);
+    if (lane == 0) prev = last;
+    last = __shfl_sync(0xffffffffu, k[j], 31);
+    nvalid += __popc(__ballot_sync(0xffffffffu, k[j] != kSentinel));
+    ballot[j] = __ballot_sync(0xffffffffu, k[j] != kSentinel && (base + j * 32 == 0 || k[j] != prev));
     wtotal += __popc(ballot[j]);
   }
   if (lane == 0) s_wsum[w] = wtotal;
   __syncthreads();
-  if (t == 0) {
+  if (w == 0) {
     uint32_t tot = 0;
     for (int ww = 0; ww < kWarps; ++ww) tot += s_wsum[ww];
     uint64_t excl = 0;
     if (tile == 0) {
       // withhold_tile0: fault-injection hook for tests; the first tile never
       // publishes, so every later tile's bounded wait runs out
-      if (!withhold_tile0) st_relaxed_u64(status, lb_word(1, kFlagInc, tot));
+      if (lane == 0 && !withhold_tile0) st_relaxed_u64(status, lb_word(1, kFlagInc, tot));
     } else {
-      st_relaxed_u64(status + tile, lb_word(1, kFlagAgg, tot));
-      excl = lookback(status, tile, 1, 1, derr);
-      st_relaxed_u64(status + tile, lb_word(1, kFlagInc, excl + tot));
+      if (lane == 0) st_relaxed_u64(status + tile, lb_word(1, kFlagAgg, tot));
+      excl = lookback_warp(status, tile, 1, lane, derr);
+      if (lane == 0) st_relaxed_u64(status + tile, lb_word(1, kFlagInc, excl + tot));
     }
-    s_excl = excl;
+    if (lane == 0) s_excl = excl;
   }
   __syncthreads();
   uint64_t o = s_excl;
   for (int ww = 0; ww < w; ++ww) o += s_wsum[ww];
 
+  // the row before the warp's first key: -1 before all keys (what precedes a
+  // valid key is valid, sentinels sorting last)
+  int32_t last_row = base - lane > 0 ? (int32_t)(before >> b) : -1;
 #pragma unroll
   for (int j = 0; j < kItems; ++j) {
     const int64_t i = base + j * 32;
     const bool keep = (ballot[j] >> lane) & 1u;
     const uint64_t my_o = o + __popc(ballot[j] & lt);
-    const uint64_t prev = prev_key(k, j, lane, i, keys, m_raw);
-    const uint64_t next = next_key(k, j, lane, i, keys, m_raw);
-    if (i < m_raw && k[j] != kSentinel) {
-      const int32_t v = (int32_t)(k[j] >> b);
+    const int32_t v = (int32_t)(k[j] >> b);
+    int32_t pv = __shfl_up_sync(0xffffffffu, v, 1);
+    if (lane == 0) pv = last_row;
+    last_row = __shfl_sync(0xffffffffu, v, 31);
+    const uint32_t at = j * 32 + lane;
+    if (at < nvalid) {
       const int32_t u = (int32_t)(k[j] & src_mask);
       if (!keep && degree_from_raw) atomicSub(&outdeg[u], 1);  // a duplicate: counted in the raw degree
       if (keep) {
         row_idx[my_o] = u;
         if (!degree_from_raw) atomicAdd(&outdeg[u], 1);
-        // rows (pv, v] start at my_o; the previous key is valid because
-        // sentinels sort last
-        const int32_t pv = (i > 0) ? (int32_t)(prev >> b) : -1;
-        if (v != pv) fill_rows(col_ptr, pv + 1, v, (int32_t)my_o, gaps, ngaps);
+        if (v != pv) fill_rows(col_ptr, pv + 1, v, (int32_t)my_o, gaps, ngaps);  // rows (pv, v] start at my_o
       }
-      if (next == kSentinel) {  // last valid key: rows (v, n] end at the total
+      // the last key of all: rows (v, n] end at the total
+      if (at + 1 == nvalid && (nvalid < kItems * 32 || i + 1 >= m_raw || keys[i + 1] == kSentinel)) {
         const int64_t total = (int64_t)my_o + (keep ? 1 : 0);
         *m_out = total;
         fill_rows(col_ptr, v + 1, n, (int32_t)total, gaps, ngaps);

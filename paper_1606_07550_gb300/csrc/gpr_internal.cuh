@@ -326,6 +326,46 @@ __device__ __forceinline__ uint64_t lookback(const uint64_t* status, int64_t til
   return excl;
 }
 
+// The same for status words one apart, by a whole warp: the words of 32
+// predecessors at once.  Every lane returns the prefix.
+__device__ __forceinline__ uint64_t lookback_warp(const uint64_t* status, int64_t tile, uint32_t epoch, int lane,
+                                                  int* derr) {
+  uint64_t excl = 0;
+  int64_t k = tile - 1;
+  uint32_t spins = 0;
+  while (k >= 0) {
+    const uint64_t w = k - lane >= 0 ? ld_relaxed_u64(status + k - lane) : 0ull;
+    const uint64_t fl = (w >> 58) & 3;
+    const bool ok = (uint32_t)(w >> 60) == epoch && fl != 0;
+    const uint32_t oks = __ballot_sync(0xffffffffu, ok);
+    const uint32_t incs = __ballot_sync(0xffffffffu, ok && fl == kFlagInc);
+    // the published words in order, up to the first inclusive one
+    int took = oks == 0xffffffffu ? 32 : __ffs(~oks) - 1;
+    const bool inc = incs != 0 && __ffs(incs) <= took;
+    if (inc) took = __ffs(incs);
+    uint64_t v = lane < took ? w & kValMask : 0ull;
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+    excl += v;
+    if (inc) break;
+    k -= took;
+    if (took == 0) {
+      if (++spins > kSpinLimit) {
+        if (lane == 0) atomicOr(derr, DERR_TIMEOUT);
+        return excl;
+      }
+      if (spins > 64) {
+        __nanosleep(64);
+        // once any waiter has given up, the rest of the grid stops waiting too
+        bool up = false;
+        if ((spins & 255) == 0) up = (*(volatile int*)derr & DERR_TIMEOUT) != 0;
+        if (__any_sync(0xffffffffu, up)) return excl;
+      }
+    }
+  }
+  return excl;
+}
+
 __device__ __forceinline__ uint32_t lanemask_lt() {
   uint32_t m;
   asm("mov.u32 %0, %%lanemask_lt;" : "=r"(m));
