@@ -976,11 +976,11 @@ static void launch_persist(const PersistArgs& A, int blocks, size_t smem, cudaSt
   count_launches(1);
 }
 
-// One product of the centralities (PersistArgs::product): no barrier, so an
-// ordinary launch.
+// One product of the centralities (kProduct): no barrier, so an ordinary
+// launch.
 static void launch_product(const PersistArgs& A, int blocks, size_t smem, cudaStream_t s) {
-  GPR_CUDA(cudaFuncSetAttribute(persist_kernel<float, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
-  persist_kernel<float, false><<<blocks, kPersThreads, smem, s>>>(A);
+  GPR_CUDA(cudaFuncSetAttribute(persist_kernel<float, false, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+  persist_kernel<float, false, true><<<blocks, kPersThreads, smem, s>>>(A);
   GPR_CUDA(cudaGetLastError());
   count_launches(1);
 }
@@ -1348,7 +1348,6 @@ gpr_status run_centrality(gpr_graph* g, int kind, int32_t iters, float* out_x, f
         A.c[1] = c_out;
         A.sums = (unsigned long long*)(w->ctl + 48) + 3 * (int64_t)products++;
         A.iters = 1;
-        A.product = 1;
         launch_product(A, ww->pers_blocks, std::max<size_t>((size_t)A.H * 4, 16), s);
       } else if (blocked)  // the contributions are held as codes
         blocked_record_step<float>(ww->blk, gg, (const uint32_t*)c_in, x_in, x_out, (uint32_t*)c_out, w->ones,
