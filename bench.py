@@ -578,7 +578,7 @@ def run_batched(args, world, rank, local):
 
     for name in args.dtypes.split(","):
         dt = dts[name]
-        # the autotuner: CTAs per cluster for each graph-size class
+        # the autotuner: step by step over the GPU, or CTAs per cluster, for each graph-size class
         tuned = gpr.ppr_tune(reqs, dtype=dt, trial_steps=8)
         for _ in range(max(1, args.warmup)):
             gpr.ppr_batch(reqs, max_iters=iters, dtype=dt)
@@ -615,7 +615,7 @@ def run_batched(args, world, rank, local):
                      "l1_max": max(l1s),
                      "l1_mean": statistics.mean(l1s), "max_rel_err_max": max(mrs), "sampled_columns": len(l1s),
                      "clocks": clk.summary(),
-                     "roofline": {"kernel": "ppr_kernel (one persistent cluster launch over every job)",
+                     "roofline": {"kernel": "ppr_rows_kernel + ppr_long_kernel (a step of every job of a wave per launch)",
                                   "bound": "hbm", "achieved": achieved, "peak": peak, "unit": "GB/s",
                                   "frac": achieved / peak, "peak_source": peak_kind,
                                   "bytes_model": "per step and job: 4m + 4(n+1) + 64n(state + s) + 64ms, state 8 (x) or "

@@ -14,8 +14,8 @@ pytestmark = pytest.mark.gpu
 EDGE = 152 * 4096  # the largest sort on the small tiles
 
 
-@pytest.mark.parametrize("n", [1, 16, 600, 70_000, 300_000])  # ids of 1, 4, 10, 17 and 19 bits
-@pytest.mark.parametrize("m", [1, 33, 4095, 4096, 4097, EDGE - 1, EDGE, EDGE + 1, 76 * 8192 + 8191, 90 * 8192 + 1])
+@pytest.mark.parametrize("n", [1, 16, 600, 300_000])  # ids of 1, 4, 10 and 19 bits
+@pytest.mark.parametrize("m", [1, 33, 4096, 4097, EDGE, EDGE + 1, 90 * 8192 + 1])
 @pytest.mark.parametrize("skewed", [False, True])
 def test_tile_edges(n, m, skewed):
     rng = np.random.default_rng(n * 7919 + m + skewed)
