@@ -21,11 +21,11 @@
 // can hold.
 //
 // What bounds it.  64 columns, FP32, 256 batch graphs (n in [1e3, 2e5], mean
-// degree 4 to 32): 270 ms for 50 steps, 8 TB/s of gathered bytes; latency-bound at
-// 24 warps an SM (80 registers; 64 registers spill and measured 302 ms), DRAM
-// 15%, L2 16-53% of peak.  On clusters (ppr.cu) the same call took 1,015 ms, 64 columns of one
-// 2^20-node graph 1,420 ms (here 28 ms) and one column of a 100,000-node graph
-// 90 ms (here 1.6 ms).
+// degree 4 to 32): 268 ms for 50 steps, 8 TB/s of gathered bytes; latency-bound at
+// 24 warps an SM (80 registers; 64 spill and measured 302 ms, 128 at 16 warps
+// 272), DRAM 21%, L2 32-47% of peak.  On clusters (ppr.cu) the same call took
+// 1,015 ms, 64 columns of one 2^20-node graph 1,420 ms (here 26 ms) and one
+// column of a 100,000-node graph 90 ms (here 1.6 ms).
 //
 // Short rows.  Two thirds of an R-MAT graph's rows have up to eight edges and
 // cost latency, not bytes: two at a time, half a warp each, took the batch
@@ -225,10 +225,24 @@ __device__ __forceinline__ void gather_warp_row(const int32_t* __restrict__ row_
         }
       };
       if constexpr (G == 2) {
-        // 16 edges in flight, or 8 where no more are left
+        // 16 edges in flight where no sums are held beside them yet, then 8 (16
+        // throughout spills 60 registers a lane, whose traffic was more than
+        // the gathers': 256 batch graphs, FP32, 274 ms against 268; 64 in BF16
+        // 94.3 against 85.2; one 2^20-node graph 28.6 against 26.0)
         int j = 0;
-        for (; j + 8 < cnt; j += 16) group(std::integral_constant<int, 8>{}, j);
-        if (j < cnt) group(std::integral_constant<int, 4>{}, j);
+        if (h == 0 && cnt > 8) {
+          float c[8][V];
+#pragma unroll
+          for (int i = 0; i < 8; ++i) ld_c<V>(base + (int64_t)__shfl_sync(0xffffffffu, idx, 2 * i + g) * stride, c[i]);
+#pragma unroll
+          for (int i = 0; i < 4; ++i)
+#pragma unroll
+            for (int v = 0; v < 2; ++v)
+              s[i][v] = add2(add2(make_float2(0.f, 0.f), make_float2(c[i][2 * v], c[i][2 * v + 1])),
+                             make_float2(c[i + 4][2 * v], c[i + 4][2 * v + 1]));
+          j = 16;
+        }
+        for (; j < cnt; j += 8) group(std::integral_constant<int, 4>{}, j);
       } else {
         if (cnt > 8)
           group(std::integral_constant<int, 4>{}, 0);
