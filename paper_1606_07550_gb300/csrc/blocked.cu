@@ -165,6 +165,8 @@ static KeyGeom key_geom(int64_t S, int64_t B, int32_t n_dense, int sb_bits) {
   return k;
 }
 
+constexpr int kStaticShared = 2048;  // static shared memory of the kernels is below this
+
 static int smem_optin() {
   int optin = 0;
   cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, device_ordinal());
@@ -190,8 +192,7 @@ bool blocked_eligible(const gpr_graph* g, int sb_bits, int w_bits) {
   if (nseg > ((int64_t)1 << 26)) return false;  // segment tables of at most 2^26 entries
   if (!geometry_fits(g, sb_bits, w_bits, 0)) return false;
   const size_t optin = (size_t)smem_optin();
-  // static shared memory of the kernels is below 2 KB
-  return expand_smem(sb_bits) + 2048 <= optin && accum_smem(w_bits) + 2048 <= optin;
+  return expand_smem(sb_bits) + kStaticShared <= optin && accum_smem(w_bits) + kStaticShared <= optin;
 }
 
 int32_t blocked_max_dense(const gpr_graph* g, int sb_bits, int w_bits) {
@@ -218,9 +219,11 @@ void blocked_free(Blocked* k, cudaStream_t s) {
   delete k;
 }
 
+// The kernel's limit is set to the most that an eligible shape asks, not to this
+// layout's: layouts of several shapes live at once.
 template <typename K>
 static int persistent_grid(K kernel, int threads, size_t smem) {
-  GPR_CUDA(cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+  GPR_CUDA(cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, smem_optin() - kStaticShared));
   int per_sm = 0;
   GPR_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kernel, threads, smem));
   return num_sms() * std::max(per_sm, 1);

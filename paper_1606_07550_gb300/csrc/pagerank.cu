@@ -953,7 +953,8 @@ static void persist_layout(gpr_graph* g, PagerankWork* w, cudaStream_t s) {
 
 template <typename T, bool kCluster>
 static void launch_persist(const PersistArgs& A, int blocks, size_t smem, cudaStream_t s) {
-  GPR_CUDA(cudaFuncSetAttribute(persist_kernel<T, kCluster>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+  // (the most of any graph: threads set it side by side)
+  GPR_CUDA(cudaFuncSetAttribute(persist_kernel<T, kCluster>, cudaFuncAttributeMaxDynamicSharedMemorySize, kPersHotBytes));
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3((unsigned)blocks, 1, 1);
   cfg.blockDim = dim3(kPersThreads, 1, 1);
@@ -979,7 +980,7 @@ static void launch_persist(const PersistArgs& A, int blocks, size_t smem, cudaSt
 // One product of the centralities (kProduct): no barrier, so an ordinary
 // launch.
 static void launch_product(const PersistArgs& A, int blocks, size_t smem, cudaStream_t s) {
-  GPR_CUDA(cudaFuncSetAttribute(persist_kernel<float, false, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+  GPR_CUDA(cudaFuncSetAttribute(persist_kernel<float, false, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, kPersHotBytes));
   persist_kernel<float, false, true><<<blocks, kPersThreads, smem, s>>>(A);
   GPR_CUDA(cudaGetLastError());
   count_launches(1);
