@@ -67,7 +67,7 @@ namespace gpr {
 constexpr int kStThreads = 32 * kStWarps;
 constexpr int32_t kLongDeg = 128;    // a batch's longer rows are summed by chunks
 constexpr int32_t kShortDeg = 8;     // rows that half a warp takes
-constexpr int kFixBits = 60;         // dangling masses and residuals are sums of multiples of 2^-60, below 8
+constexpr int kFixBits = 60;         // dangling masses and residuals are sums of multiples of 2^-60, within 8 of 0
 
 // Edges per chunk of a row of deg edges, more than long_deg: long_deg, or about
 // sqrt(2 deg), since the chunk sums of one row are added by one warp.
@@ -77,13 +77,21 @@ __host__ __device__ __forceinline__ int32_t chunk_edges(int32_t deg, int32_t lon
   return c;
 }
 
-// v * 2^kFixBits, truncated (0 <= v < 8), from the bits of v: a conversion
-// instruction to 64 bits would run on the slow FP64 pipe.
+// v * 2^kFixBits, truncated (-8 < v < 8), in two's complement, from the bits of
+// v: a conversion instruction to 64 bits would run on the slow FP64 pipe.  A
+// dangling mass can be below zero: what a row has sent as BF16 deltas passes its
+// contribution by up to 2^-9 of the last delta, and where x falls to less than
+// that in a step (a cycle's front passing, d above 0.998) the rows after it
+// have x < 0 for one step.
 __device__ __forceinline__ unsigned long long fix_of(float v) {
   const uint32_t u = __float_as_uint(v);
-  const int sh = (int)(u >> 23) - 150 + kFixBits;
+  const int sh = (int)((u >> 23) & 0xFFu) - 150 + kFixBits;
   const unsigned long long f = (u & 0x7FFFFFu) | 0x800000u;
-  return sh >= 0 ? f << min(sh, 40) : sh > -24 ? f >> -sh : 0ull;
+  const unsigned long long a = sh >= 0 ? f << min(sh, 40) : sh > -24 ? f >> -sh : 0ull;
+  return (int32_t)u < 0 ? 0ull - a : a;
+}
+__device__ __forceinline__ double fix_value(unsigned long long a) {
+  return (double)(long long)a * (1.0 / (double)(1ull << kFixBits));
 }
 
 template <int W>
@@ -770,8 +778,7 @@ __global__ void __launch_bounds__(kStThreads, 3) ppr_rows_kernel(const StepJob* 
   __threadfence();
   int live = 0;
   if (tid < W && cs.live[tid]) {
-    constexpr double unit = 1.0 / (double)(1ull << kFixBits);
-    const double D = (double)__ldcg(&st->acc[0][tid]) * unit, res = (double)__ldcg(&st->acc[1][tid]) * unit;
+    const double D = fix_value(__ldcg(&st->acc[0][tid])), res = fix_value(__ldcg(&st->acc[1][tid]));
     st->acc[0][tid] = st->acc[1][tid] = 0ull;
     const double d = cs.d[tid];
     const int32_t it = st->iters[tid] + 1;

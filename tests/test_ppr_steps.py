@@ -98,3 +98,22 @@ def test_columns_that_stop_at_different_steps(case):
         xr, k_ref = oracle.ppr(ref, int(seeds[j]), 0.85, 200, 1e-4)
         assert abs(int(it[j]) - k_ref) <= 1 and 0.85 / 0.15 * res[j] <= 1e-4 * (1 + 1e-3)
         assert l1(x[:, j], oracle.ppr(ref, int(seeds[j]), 0.85, 300)[0]) <= 1e-4 + 1e-5
+
+
+@pytest.mark.gpu
+@pytest.mark.parametrize("k", [1, 3, 16, 64])
+def test_bf16_rows_below_zero(k):
+    # a cycle with a chord and a dangling node after node 4: as the front passes,
+    # x[4] falls by a factor of a thousand in one step, the rounding of the sent
+    # delta overshoots it, and the dangling mass is below zero at steps 12 (from
+    # node 0) and 9 (from node 3).  A step's rounding moves at most 2^-9 of
+    # ||x_k - x_{k-1}||_1 <= 2 (and of the rounding before), so 30 steps are
+    # within 30 * 2.01 * 2^-9 of the exact ones
+    import torch
+    src, dst = np.array([0, 1, 2, 3, 4, 4, 3], np.int32), np.array([1, 2, 3, 4, 0, 5, 1], np.int32)
+    g, ref = gpr.graph_build(src, dst, 6), oracle.build_csc(6, src, dst)
+    seeds = np.resize(np.array([0, 3], np.int32), k)
+    x = torch.zeros((6, k), dtype=torch.float32, device="cuda")
+    gpr.ppr_batch([(g, seeds, 0.999, x)], max_iters=30, dtype=gpr.BF16)
+    for j in range(min(k, 2)):
+        assert l1(x[:, j].cpu().numpy(), oracle.ppr(ref, int(seeds[j]), 0.999, 30)[0]) <= 0.12
