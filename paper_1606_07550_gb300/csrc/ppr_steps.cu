@@ -979,7 +979,9 @@ __global__ void __launch_bounds__(kStThreads) ppr_start_kernel(const StepJob* __
 }
 
 // The same for the columns that have joined a server's slot (status kColFresh
-// in its records) since its last steps; those that finished then leave.
+// in its records) since its last steps; those that finished then leave, and so
+// do those whose record says that they are gone: the records are the server's
+// word, the state is this side's.
 template <typename T>
 __global__ void __launch_bounds__(kStThreads) ppr_join_kernel(const StepJob* __restrict__ jobs,
                                                              const StepItem* __restrict__ items) {
@@ -990,10 +992,11 @@ __global__ void __launch_bounds__(kStThreads) ppr_join_kernel(const StepJob* __r
   const StepItem item = items[blockIdx.x];
   const StepJob* J = jobs + item.slot;
   const int tid = threadIdx.x;
-  int fresh = 0;
+  int fresh = 0, going = 0;
   if (tid < W) {
     const PprCol c = J->cols[tid];
     fresh = c.status == kColFresh;
+    going = c.status == kColRunning;
     s_fresh[tid] = (uint8_t)fresh;
     s_seed[tid] = fresh ? J->old2new[c.seed] : -1;
   }
@@ -1003,7 +1006,7 @@ __global__ void __launch_bounds__(kStThreads) ppr_join_kernel(const StepJob* __r
     if (tid < W) {
       if (fresh)
         live = start_column(J, J->cols[tid], tid);
-      else if (st->status[tid] == kColRunning)
+      else if (going && st->status[tid] == kColRunning)
         live = 1;
       else
         st->status[tid] = kColEmpty;

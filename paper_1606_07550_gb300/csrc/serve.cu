@@ -24,6 +24,7 @@
 #include <chrono>
 #include <climits>
 #include <condition_variable>
+#include <cstdlib>
 #include <deque>
 #include <thread>
 #include <unordered_map>
@@ -97,6 +98,7 @@ struct gpr_server {
   bool stop = false;
   std::thread th;
   int alloc_attempts = 0;
+  int fail_tick = 0;  // test hook (GPR_INJECT_TICK_FAILURE): this tick has no memory for its items
   gpr_server_stats st{};
   // device staging for one tick
   gpr::StepJob* d_desc = nullptr;
@@ -275,12 +277,17 @@ static bool try_admit(gpr_server* S, Req& r, bool existing_only = false) {
   return true;
 }
 
+// Room for `need` entries (fail: as if there were no memory for them).
 template <typename V>
-static V* grow(V* p, int& cap, int need, cudaStream_t s) {
-  if (need <= cap) return p;
+static void grow(V*& p, int& cap, int need, cudaStream_t s, bool fail = false) {
+  if (need <= cap && !fail) return;
   dfree(p, s);
-  cap = std::max(need, 2 * cap + 16);
-  return (V*)dalloc((size_t)cap * sizeof(V), s);
+  p = nullptr;
+  const int want = std::max(need, 2 * cap + 16);
+  cap = 0;
+  if (fail) throw StatusFail{GPR_ENOMEM, "injected allocation failure"};
+  p = (V*)dalloc((size_t)want * sizeof(V), s);
+  cap = want;
 }
 
 // One tick: per storage type, steps_per_tick steps of every item of the slots
@@ -293,7 +300,7 @@ static void run_tick(gpr_server* S, const std::vector<Slot*>& live) {
     fill_desc(desc[i], S, sl);
     GPR_CUDA(cudaMemcpyAsync(sl->d_rec, sl->cols, kPprCols * sizeof(PprCol), cudaMemcpyHostToDevice, S->stream));
   }
-  S->d_desc = grow(S->d_desc, S->cap_desc, (int)desc.size(), S->stream);
+  grow(S->d_desc, S->cap_desc, (int)desc.size(), S->stream);
   GPR_CUDA(cudaMemcpyAsync(S->d_desc, desc.data(), desc.size() * sizeof(StepJob), cudaMemcpyHostToDevice, S->stream));
   const int32_t T = S->cfg.steps_per_tick;
   for (gpr_dtype dt : {GPR_FP32, GPR_BF16, GPR_FP16}) {
@@ -308,11 +315,11 @@ static void run_tick(gpr_server* S, const std::vector<Slot*>& live) {
     }
     if (items.empty()) continue;
     const int32_t ni = (int32_t)items.size(), nci = (int32_t)citems.size();
-    S->d_items = grow(S->d_items, S->cap_items, ni, S->stream);
+    grow(S->d_items, S->cap_items, ni, S->stream, S->fail_tick > 0 && S->st.ticks + 1 == S->fail_tick);
     GPR_CUDA(cudaMemcpyAsync(S->d_items, items.data(), items.size() * sizeof(StepItem), cudaMemcpyHostToDevice,
                              S->stream));
     if (nci > 0) {
-      S->d_citems = grow(S->d_citems, S->cap_citems, nci, S->stream);
+      grow(S->d_citems, S->cap_citems, nci, S->stream);
       GPR_CUDA(cudaMemcpyAsync(S->d_citems, citems.data(), citems.size() * sizeof(StepItem),
                                cudaMemcpyHostToDevice, S->stream));
     }
@@ -326,6 +333,10 @@ static void run_tick(gpr_server* S, const std::vector<Slot*>& live) {
   for (Slot* sl : live) sl->parity = (sl->parity + T) & 1;
 }
 
+// After a failed tick: every running request fails, and its slot goes with it,
+// since nobody knows how far the device's column state has come.  (The results
+// stay until serve_release; what the tick has queued is ahead of their release
+// on the stream.)
 static void fail_running(gpr_server* S, gpr_status st) {
   for (Slot* sl : S->slots) {
     for (int c = 0; c < kPprCols; ++c) {
@@ -338,11 +349,10 @@ static void fail_running(gpr_server* S, gpr_status st) {
         ++S->st.failed;
         S->finished.push_back(it->first);
       }
-      sl->owner[c] = 0;
-      sl->cols[c].status = kColEmpty;
     }
-    sl->used = 0;
+    free_slot(S, sl);
   }
+  S->slots.clear();
   S->cv_done.notify_all();
 }
 
@@ -469,6 +479,7 @@ gpr_status serve_create(const gpr_graph* const* pool, int32_t num_graphs, const 
   S->cfg = *cfg;
   if (S->cfg.max_queue <= 0) S->cfg.max_queue = 65536;
   if (S->cfg.steps_per_tick <= 0) S->cfg.steps_per_tick = 8;
+  if (const char* e = getenv("GPR_INJECT_TICK_FAILURE")) S->fail_tick = atoi(e);
   std::vector<const gpr_graph*> uniq(S->pool);
   std::sort(uniq.begin(), uniq.end());
   uniq.erase(std::unique(uniq.begin(), uniq.end()), uniq.end());
