@@ -366,6 +366,24 @@ __device__ __forceinline__ uint64_t lookback_warp(const uint64_t* status, int64_
   return excl;
 }
 
+// Sums of multiples of 2^-60, exact in any order: v * 2^60, truncated (0 <= v < 8;
+// fix60_signed: -8 < v < 8, in two's complement), from the bits of v: a conversion
+// instruction to 64 bits would run on the slow FP64 pipe.
+constexpr int kFixBits = 60;
+__device__ __forceinline__ unsigned long long fix60(float v) {
+  const uint32_t u = __float_as_uint(v);
+  const int sh = (int)(u >> 23) - 150 + kFixBits;
+  const unsigned long long f = (u & 0x7FFFFFu) | 0x800000u;
+  return sh >= 0 ? f << min(sh, 40) : sh > -24 ? f >> -sh : 0ull;
+}
+__device__ __forceinline__ unsigned long long fix60_signed(float v) {
+  const unsigned long long a = fix60(fabsf(v));
+  return v < 0.f ? 0ull - a : a;
+}
+__device__ __forceinline__ double fix60_value(unsigned long long a) {
+  return (double)(long long)a * (1.0 / (double)(1ull << kFixBits));
+}
+
 __device__ __forceinline__ uint32_t lanemask_lt() {
   uint32_t m;
   asm("mov.u32 %0, %%lanemask_lt;" : "=r"(m));

@@ -45,7 +45,11 @@
 // taken this way, in order.  The dangling mass and the residual are FP32 sums
 // over the rows of a piece (about kPieceWork units of work), 32 rows at a time,
 // the short rows (up to kShortDeg edges) before the others, each in row order;
-// then exact integer sums of those in units of 2^-kFixBits, in any order.
+// then exact integer sums of those in units of 2^-60, in any order (a dangling
+// mass can be below zero: what a row has sent as BF16 deltas passes its
+// contribution by up to 2^-9 of the last delta, and where x falls to less than
+// that in a step, a cycle's front passing with d above 0.998, the rows after it
+// have x < 0 for one step).
 //
 // The server (serve.cu) runs its slots' steps on the same kernels, 64 columns
 // wide.
@@ -67,7 +71,6 @@ namespace gpr {
 constexpr int kStThreads = 32 * kStWarps;
 constexpr int32_t kLongDeg = 128;    // a batch's longer rows are summed by chunks
 constexpr int32_t kShortDeg = 8;     // rows that half a warp takes
-constexpr int kFixBits = 60;         // dangling masses and residuals are sums of multiples of 2^-60, within 8 of 0
 
 // Edges per chunk of a row of deg edges, more than long_deg: long_deg, or about
 // sqrt(2 deg), since the chunk sums of one row are added by one warp.
@@ -75,23 +78,6 @@ __host__ __device__ __forceinline__ int32_t chunk_edges(int32_t deg, int32_t lon
   int32_t c = long_deg;
   while (deg / c >= 2 * c) c *= 2;
   return c;
-}
-
-// v * 2^kFixBits, truncated (-8 < v < 8), in two's complement, from the bits of
-// v: a conversion instruction to 64 bits would run on the slow FP64 pipe.  A
-// dangling mass can be below zero: what a row has sent as BF16 deltas passes its
-// contribution by up to 2^-9 of the last delta, and where x falls to less than
-// that in a step (a cycle's front passing, d above 0.998) the rows after it
-// have x < 0 for one step.
-__device__ __forceinline__ unsigned long long fix_of(float v) {
-  const uint32_t u = __float_as_uint(v);
-  const int sh = (int)((u >> 23) & 0xFFu) - 150 + kFixBits;
-  const unsigned long long f = (u & 0x7FFFFFu) | 0x800000u;
-  const unsigned long long a = sh >= 0 ? f << min(sh, 40) : sh > -24 ? f >> -sh : 0ull;
-  return (int32_t)u < 0 ? 0ull - a : a;
-}
-__device__ __forceinline__ double fix_value(unsigned long long a) {
-  return (double)(long long)a * (1.0 / (double)(1ull << kFixBits));
 }
 
 template <int W>
@@ -755,8 +741,8 @@ __global__ void __launch_bounds__(kStThreads, 3) ppr_rows_kernel(const StepJob* 
     if (lane < L) {
 #pragma unroll
       for (int v = 0; v < V; ++v) {
-        s_acc[warp][0][c0 + v] += fix_of(dsum[v]);
-        s_acc[warp][1][c0 + v] += fix_of(rsum[v]);
+        s_acc[warp][0][c0 + v] += fix60_signed(dsum[v]);
+        s_acc[warp][1][c0 + v] += fix60(rsum[v]);
       }
     }
   }
@@ -778,7 +764,7 @@ __global__ void __launch_bounds__(kStThreads, 3) ppr_rows_kernel(const StepJob* 
   __threadfence();
   int live = 0;
   if (tid < W && cs.live[tid]) {
-    const double D = fix_value(__ldcg(&st->acc[0][tid])), res = fix_value(__ldcg(&st->acc[1][tid]));
+    const double D = fix60_value(__ldcg(&st->acc[0][tid])), res = fix60_value(__ldcg(&st->acc[1][tid]));
     st->acc[0][tid] = st->acc[1][tid] = 0ull;
     const double d = cs.d[tid];
     const int32_t it = st->iters[tid] + 1;

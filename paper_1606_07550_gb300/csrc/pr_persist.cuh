@@ -23,9 +23,12 @@
 // SMs.)  Longer rows go round-robin to blocks, which cut them into chunks for
 // their warps and add a row's chunk sums after a block barrier.
 //
-// Mass, dangling mass and residual: FP32 per thread and warp as in the pull
-// kernels, then exact integer sums of multiples of 2^-60 over warps and blocks,
-// so runs are bitwise identical.
+// Mass, dangling mass and residual: FP32 per thread and over the warp as in the
+// pull kernels, then exact integer sums of multiples of 2^-60 over warps and
+// blocks, so runs are bitwise identical.  A thread has more rows here, and where
+// most rows hold the same rank all threads round alike, so its mass and dangling
+// mass are sums of two floats (2^20 nodes and edges: L1 error 3.3e-8; with plain
+// sums 6.4e-8, with the pull kernels 3.5e-8; times within 1.5% either way).
 //
 // The centralities take the same kernel a step at a time (kProduct):
 // one launch a product instead of six.
@@ -74,14 +77,6 @@ struct PersistArgs {
   int32_t iters;
 };
 
-constexpr int kPersFix = 60;
-__device__ __forceinline__ unsigned long long pers_fix(float v) {  // v * 2^60 truncated, 0 <= v < 8
-  const uint32_t u = __float_as_uint(v);
-  const int sh = (int)(u >> 23) - 150 + kPersFix;
-  const unsigned long long f = (u & 0x7FFFFFu) | 0x800000u;
-  return sh >= 0 ? f << min(sh, 40) : sh > -24 ? f >> -sh : 0ull;
-}
-
 // The stored contribution of source u: from the shared-memory copy of the first
 // H, from L2 above, 0 for u < 0.  Predicated loads, no branch: a warp's loads
 // overlap whichever way its lanes go.  The bits, to be taken by pers_value once
@@ -113,7 +108,7 @@ __device__ __forceinline__ float2 pers_pair(unsigned long long s) {
   // 24 bits from the leading one on, and the rest
   const int z = __clzll((long long)(s | 1ull)), sh = 40 - z;
   const unsigned long long hi = sh > 0 ? (s >> sh) << sh : s;
-  const float a = (float)(uint32_t)(sh > 0 ? s >> sh : s), unit = __uint_as_float((uint32_t)(127 - kPersFix) << 23);
+  const float a = (float)(uint32_t)(sh > 0 ? s >> sh : s), unit = __uint_as_float((uint32_t)(127 - kFixBits) << 23);
   const float scale = sh > 0 ? __uint_as_float((uint32_t)(127 + sh) << 23) : 1.0f;
   const unsigned long long lo = s - hi;  // below 2^40
   const float b = fmaf((float)(uint32_t)(lo >> 16), 65536.0f, (float)(uint32_t)(lo & 0xFFFFu));
@@ -193,16 +188,8 @@ __global__ void __launch_bounds__(kPersThreads, 1) persist_kernel(const __grid_c
       failed = s_bad != 0;
     }
   };
-  // this thread's part of the step's sums into row `it`
-  auto add_sums = [&](int32_t it, float mass, float dang, float res) {
-    mass = warp_sum(mass);
-    dang = warp_sum(dang);
-    res = warp_sum(res);
-    if (lane == 0) {
-      s_sum[0][warp] = pers_fix(mass);
-      s_sum[1][warp] = pers_fix(dang);
-      s_sum[2][warp] = pers_fix(res);
-    }
+  // the block's sums into row `it`
+  auto add_sums = [&](int32_t it) {
     __syncthreads();
     if (warp < 3) {
       unsigned long long t = lane < kPersWarps ? s_sum[warp][lane] : 0ull;
@@ -216,7 +203,6 @@ __global__ void __launch_bounds__(kPersThreads, 1) persist_kernel(const __grid_c
     for (int o = 16; o > 0; o >>= 1) mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, o));
     if (lane == 0 && mx > 0.f) atomicMax((unsigned int*)(A.sums + 3 * (int64_t)it), __float_as_uint(mx));
   };
-  constexpr double unit = 1.0 / (double)(1ull << kPersFix);
 
   // the block's long rows and their chunks
   for (int32_t j = tid; j < nl; j += kPersThreads) s_span[j] = A.span[my_long[j]];
@@ -255,15 +241,22 @@ __global__ void __launch_bounds__(kPersThreads, 1) persist_kernel(const __grid_c
   const float x0 = 1.0f / (float)n;
   if constexpr (!kProduct) {
     T* c0 = (T*)A.c[0];
-    float mass = 0.f, dang = 0.f;
+    int32_t rows = 0, ends = 0;  // of the thread, without out-edges
     for (int32_t v = blockIdx.x * kPersThreads + tid; v < n; v += nblk * kPersThreads) {
       const float idg = A.inv_deg[v];
       store_rank(c0, v, x0 * idg);
       if (A.iters == 0) A.x[v] = x0;
-      mass += x0;
-      if (idg == 0.f) dang += x0;
+      ++rows;
+      if (idg == 0.f) ++ends;
     }
-    add_sums(0, mass, dang, 0.f);
+    rows = __reduce_add_sync(0xffffffffu, rows);
+    ends = __reduce_add_sync(0xffffffffu, ends);
+    if (lane == 0) {
+      s_sum[0][warp] = fix60(x0) * (unsigned)rows;
+      s_sum[1][warp] = fix60(x0) * (unsigned)ends;
+      s_sum[2][warp] = 0ull;
+    }
+    add_sums(0);
   }
   if constexpr (kProduct) __syncthreads();  // (add_sums has one)
   const int32_t nchunks = s_first[nl];
@@ -338,15 +331,23 @@ __global__ void __launch_bounds__(kPersThreads, 1) persist_kernel(const __grid_c
     }
     __syncthreads();
     const float ca = s_coef[0], cb = s_coef[1];
-    float mass = 0.f, dang = 0.f, res = 0.f;
+    float mass = 0.f, dang = 0.f, res = 0.f, mass_c = 0.f, dang_c = 0.f;
+    auto two = [](float& s, float& c, float v) {  // s + c += v
+      const float t = s + v, b = t - s;
+      c += (s - (t - b)) + (v - b);
+      s = t;
+    };
     auto finish = [&](int32_t i, int32_t r, float inv, float xo, float y) {
       const float xs = fmaf(ca, y, cb);
       A.xi[i] = xs;
       if (last) A.x[r] = xs;
       if (!last || kProduct) store_rank(cout, r, xs * inv);
-      mass = kProduct ? fmaxf(mass, xs) : mass + xs;
+      if constexpr (kProduct)
+        mass = fmaxf(mass, xs);
+      else
+        two(mass, mass_c, xs);
       res += fabsf(xs - xo);
-      if (inv == 0.0f) dang += xs;
+      if (inv == 0.0f) two(dang, dang_c, xs);
       return xs;
     };
     auto gather = [&](const auto& u) {
@@ -425,25 +426,54 @@ __global__ void __launch_bounds__(kPersThreads, 1) persist_kernel(const __grid_c
     }
     if (nl > 0) {
       __syncthreads();
-      if (tid < nl) {
-        float y = 0.f;
-        for (int32_t q = s_first[tid]; q < s_first[tid + 1]; ++q) y += s_chunk[q];
-        const int32_t i = __ldg(my_long + tid);
-        finish(i, __ldg(A.row + i), __ldg(A.inv + i), it > 0 ? A.xi[i] : x0, y);
+      if (32 * warp < nl) {
+        const bool mine = tid < nl;
+        int32_t i = 0, r = 0, q = 0, q1 = 0;
+        float inv = 0.f, xo = x0, y = 0.f;
+        if (mine) {
+          i = __ldg(my_long + tid);
+          r = __ldg(A.row + i);
+          inv = __ldg(A.inv + i);
+          if (it > 0) xo = A.xi[i];
+          q = s_first[tid];
+          q1 = s_first[tid + 1];
+        }
+        for (; q < q1; ++q) y += s_chunk[q];
+        // (rows have different numbers of chunks: without this the lanes of each
+        // number may finish by themselves, one number after another, which took
+        // 10 us of a step)
+        __syncwarp();
+        if (mine) finish(i, r, inv, xo, y);
       }
     }
     if constexpr (kProduct) {
       add_max(it + 1, mass);
       return;
     }
-    add_sums(it + 1, mass, dang, res);
+    mass = warp_sum(mass);
+    dang = warp_sum(dang);
+    res = warp_sum(res);
+    if (lane == 0) {
+      s_sum[0][warp] = fix60(mass);
+      s_sum[1][warp] = fix60(dang);
+      s_sum[2][warp] = fix60(res);
+    }
+    if (!single) {
+      mass_c = warp_sum(mass_c);
+      dang_c = warp_sum(dang_c);
+      if (lane == 0) {
+        s_sum[0][warp] += fix60_signed(mass_c);
+        s_sum[1][warp] += fix60_signed(dang_c);
+      }
+    }
+    add_sums(it + 1);
     barrier();
   }
 
   // ranks by caller id; x_0 of a call without steps was written above
   for (int32_t v = blockIdx.x * kPersThreads + tid; v < n; v += nblk * kPersThreads)
     A.out[v] = failed ? __int_as_float(0x7fffffff) : __ldcg(A.x + A.old2new[v]);
-  if (blockIdx.x == 0 && tid < 3) A.log_row[tid] = (double)__ldcg(A.sums + 3 * (int64_t)A.iters + tid) * unit;
+  if (blockIdx.x == 0 && tid < 3) A.log_row[tid] = fix60_value(__ldcg(A.sums + 3 * (int64_t)A.iters + tid));
 }
 
 // ---- the layout -------------------------------------------------------------

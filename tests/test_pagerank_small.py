@@ -79,3 +79,17 @@ def test_other_damping_and_two_graphs_in_turn():
             outs.append(x)
         for (g, ref), x in zip(graphs * 2, outs):
             assert l1(x.cpu().numpy(), oracle.pagerank(ref, d, 30)) <= 1e-5
+
+
+@pytest.mark.parametrize("n", [700_001, 1_300_003])
+def test_sums_over_many_equal_rows(n):
+    # All ranks but two are equal: a lane's two-float sum is exact to 2^-45 of
+    # itself, the warp trees of equal numbers are exact, the two warps with other
+    # ranks round by 5 * 2^-24 of their 20 * 32 / n of the mass, and 2^-60 is cut
+    # off in each of 2 * 3,648 places: below 1e-9 together
+    import torch
+    g = gpr.graph_build(np.array([5], np.int32), np.array([9], np.int32), n)
+    for iters in (0, 1, 3):
+        x, st = run(torch, g, iters, gpr.FP32, stats=True)
+        x = x.astype(np.float64)
+        assert abs(st.mass - x.sum()) <= 1e-9 and abs(st.dangling - (x.sum() - x[5])) <= 1e-9
