@@ -779,10 +779,22 @@ static Choice pick(gpr_graph* g, PagerankWork* w, int flags, gpr_dtype dt, cudaS
 // Whether the call takes it: the pull schedule of a graph below kTuneMinEdges
 // from the uniform vector, without the hot pass.  (A warm start's vector need
 // not sum to about one, as the kernel's fixed-point sums want it.)
-static bool persist_eligible(const gpr_graph* g, const PagerankWork* w, int sched, bool warm) {
+//
+// A warp does its slices of 32 rows one after another, so rows cost more here
+// than in the pull kernels, and edges and launches less.  From 1.5 M rows on every
+// further row has to bring an edge; us of 50 FP32 steps, pull kernels / here:
+// 1.25 M rows and 2^12 edges 809 / 782, 1.5 M and 2^12 831 / 906, 2^18 1,022 / 928;
+// 2 M and 2^18 1,075 / 1,089, 2^19 1,147 / 1,104; 3 M and 2^20 1,536 / 1,639, 3 2^19
+// 1,723 / 1,648; 4 M and 3 2^19 2,271 / 2,286, 2^21 2,534 / 2,215; 8 M and 2^22
+// 5,094 / 6,348.  The centralities' products have no barrier and cost less a row:
+// 10 steps of HITS on 8 M rows and 2^15 edges 1,970 / 1,889, on 16 M and 2^20
+// 3,319 / 3,675.
+constexpr int32_t kPersMaxRows = 1 << 22, kPersFreeRows = 3 << 19, kProductMaxRows = 1 << 23;
+static bool persist_eligible(const gpr_graph* g, const PagerankWork* w, int sched, bool warm, bool product = false) {
   // a block's long rows fit its lists: at most m / 65 rows, dealt out evenly
   static_assert(kTuneMinEdges / (kPersShort + 1) / 128 < kPersLongRows, "long rows of a block");
-  return sched == kSchedPull && !warm && w->hot_grid == 0 && g->m < kTuneMinEdges && num_sms() >= 128;
+  const bool rows = product ? g->n <= kProductMaxRows : g->n <= kPersMaxRows && g->n <= kPersFreeRows + g->m;
+  return sched == kSchedPull && !warm && w->hot_grid == 0 && g->m < kTuneMinEdges && rows && num_sms() >= 128;
 }
 
 // Contributions kept in shared memory, in bytes: all of a graph's, or the
@@ -1330,8 +1342,8 @@ gpr_status run_centrality(gpr_graph* g, int kind, int32_t iters, float* out_x, f
     }
     // small graphs: the products of the single-launch kernel, each a launch of
     // its own (ones as inverse degrees: pers_inv is PageRank's)
-    const bool small = !blocked && persist_eligible(g, w, kSchedPull, false) &&
-                       (kind == 0 || persist_eligible(t, wt, kSchedPull, false));
+    const bool small = !blocked && persist_eligible(g, w, kSchedPull, false, true) &&
+                       (kind == 0 || persist_eligible(t, wt, kSchedPull, false, true));
     if (small) {
       if (!w->pers) persist_layout(g, w, s);
       if (kind == 1 && !wt->pers) persist_layout(t, wt, s);

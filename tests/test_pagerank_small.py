@@ -93,3 +93,28 @@ def test_sums_over_many_equal_rows(n):
         x, st = run(torch, g, iters, gpr.FP32, stats=True)
         x = x.astype(np.float64)
         assert abs(st.mass - x.sum()) <= 1e-9 and abs(st.dangling - (x.sum() - x[5])) <= 1e-9
+
+
+@pytest.mark.parametrize("n,m,one", [((3 << 19) + 100, 100, True), ((3 << 19) + 101, 100, False),
+                                     (1 << 22, 3 << 20, True), ((1 << 22) + 1, 3 << 20, False)])
+def test_lines_of_the_single_launch(n, m, one):
+    # many rows for their edges: on both sides of the rule's lines, one launch a
+    # call or the pull kernels, and the same ranks
+    import torch
+    gen = torch.Generator(device="cuda").manual_seed(n)
+    dst = torch.randperm(n, dtype=torch.int32, device="cuda", generator=gen)[:m]  # m distinct edges
+    g = gpr.graph_build((dst + 1) % n, dst, n)
+    assert g.info().m == m
+    x, _ = run(torch, g, 20, gpr.FP32)
+    before = gpr.lib().gpr_kernel_launches()
+    again, _ = run(torch, g, 20, gpr.FP32)
+    assert (gpr.lib().gpr_kernel_launches() - before == 1) == one
+    assert (again == x).all()
+    y, _ = run(torch, g, 20, gpr.FP32, warm=True)
+    assert l1(x, y) <= 2 * tolerance(gpr.FP32, 20)
+    h, a = (torch.empty(n, device="cuda") for _ in range(2))
+    gpr.hits(g, h, a, iters=2, spmv="pull")
+    # an edge's head has one in-edge, its tail one out-edge: all hubs and authorities alike
+    want = torch.zeros(n, device="cuda")
+    want[dst.long()] = m ** -0.5
+    assert float((a - want).norm()) <= 1e-5 and float((h - want.roll(1)).norm()) <= 1e-5
