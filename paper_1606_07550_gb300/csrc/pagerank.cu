@@ -674,22 +674,41 @@ static void ensure_exec(gpr_graph* g, PagerankWork* w, int32_t iters, gpr_dtype 
                                            : 2 + (int64_t)iters * (g->plan.nbuckets + 1 + (w->hot_grid > 0 ? 1 : 0));
 }
 
-// Device time of `iters` steps of schedule c, after one untimed run.
+// The iteration of a small graph in one launch (below).
+static bool persist_eligible(const gpr_graph* g, const PagerankWork* w, int sched, bool warm, bool product = false);
+static void persist_prepare(gpr_graph* g, PagerankWork* w, cudaStream_t s);
+static void persist_run(gpr_graph* g, PagerankWork* w, double damping, int32_t iters, gpr_dtype dt, float* dst,
+                        cudaStream_t s);
+static void check_persist(PagerankWork* w, cudaStream_t s);
+
+// Device time of `iters` steps of schedule c as a call would run them, after one
+// untimed run.
 static double time_choice(gpr_graph* g, PagerankWork* w, const Choice& c, int32_t iters, gpr_dtype dt,
                           cudaStream_t s) {
-  if (c.sched == kSchedBlocked) ensure_layout(g, w, c, s);
-  ensure_exec(g, w, iters, dt, c.sched, false, s);
+  const bool persist = persist_eligible(g, w, c.sched, false);
+  if (persist) {
+    persist_prepare(g, w, s);
+    if (!w->out_tmp) w->out_tmp = (float*)dalloc((size_t)g->n * 4, s);
+  } else {
+    if (c.sched == kSchedBlocked) ensure_layout(g, w, c, s);
+    ensure_exec(g, w, iters, dt, c.sched, false, s);
+  }
   const StepParams hp{0.f, 0.f, 0.85, (double)g->n};
   float best = 0.f;
   for (int rep = 0; rep < 2; ++rep) {
     GPR_CUDA(cudaMemcpyAsync(w->prm, &hp, sizeof hp, cudaMemcpyHostToDevice, s));
     GPR_CUDA(cudaEventRecord(w->ev_t0, s));
-    GPR_CUDA(cudaGraphLaunch(w->exec, s));
+    if (persist) {
+      persist_run(g, w, hp.d, iters, dt, w->out_tmp, s);
+    } else {
+      GPR_CUDA(cudaGraphLaunch(w->exec, s));
+      count_launches(w->exec_kernels);
+    }
     GPR_CUDA(cudaEventRecord(w->ev_t1, s));
-    count_launches(w->exec_kernels);
     GPR_CUDA(cudaStreamSynchronize(s));
     GPR_CUDA(cudaEventElapsedTime(&best, w->ev_t0, w->ev_t1));
   }
+  if (persist) check_persist(w, s);
   return best;
 }
 
@@ -790,7 +809,7 @@ static Choice pick(gpr_graph* g, PagerankWork* w, int flags, gpr_dtype dt, cudaS
 // 10 steps of HITS on 8 M rows and 2^15 edges 1,970 / 1,889, on 16 M and 2^20
 // 3,319 / 3,675.
 constexpr int32_t kPersMaxRows = 1 << 22, kPersFreeRows = 3 << 19, kProductMaxRows = 1 << 23;
-static bool persist_eligible(const gpr_graph* g, const PagerankWork* w, int sched, bool warm, bool product = false) {
+static bool persist_eligible(const gpr_graph* g, const PagerankWork* w, int sched, bool warm, bool product) {
   // a block's long rows fit its lists: at most m / 65 rows, dealt out evenly
   static_assert(kTuneMinEdges / (kPersShort + 1) / 128 < kPersLongRows, "long rows of a block");
   const bool rows = product ? g->n <= kProductMaxRows : g->n <= kPersMaxRows && g->n <= kPersFreeRows + g->m;
@@ -1058,6 +1077,22 @@ static void run_persist(gpr_graph* g, PagerankWork* w, double damping, int32_t i
     launch_persist<T, false>(A, w->pers_blocks, smem, s);
 }
 
+static void persist_prepare(gpr_graph* g, PagerankWork* w, cudaStream_t s) {
+  // (a stream being captured cannot take the graph launch of the other way either)
+  cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+  GPR_CUDA(cudaStreamIsCapturing(s, &cap));
+  if (cap != cudaStreamCaptureStatusNone) throw CudaFail{cudaErrorStreamCaptureUnsupported, "pagerank"};
+  if (!w->pers) persist_layout(g, w, s);
+}
+
+static void persist_run(gpr_graph* g, PagerankWork* w, double damping, int32_t iters, gpr_dtype dt, float* dst,
+                        cudaStream_t s) {
+  if (dt == GPR_BF16)
+    run_persist<__nv_bfloat16>(g, w, damping, iters, dst, s);
+  else
+    run_persist<float>(g, w, damping, iters, dst, s);
+}
+
 // Whether the launch's barrier gave up (a call that does not synchronise sees
 // NaN ranks instead).
 static void check_persist(PagerankWork* w, cudaStream_t s) {
@@ -1097,11 +1132,7 @@ gpr_status run_pagerank(gpr_graph* g, double damping, int32_t iters, gpr_dtype d
     }
     const bool persist = persist_eligible(g, w, sched, warm);
     if (persist) {
-      // (a stream being captured cannot take the graph launch of the other way either)
-      cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
-      GPR_CUDA(cudaStreamIsCapturing(s, &cap));
-      if (cap != cudaStreamCaptureStatusNone) throw CudaFail{cudaErrorStreamCaptureUnsupported, "pagerank"};
-      if (!w->pers) persist_layout(g, w, s);
+      persist_prepare(g, w, s);
     } else {
       ensure_exec(g, w, iters, dt, sched, warm, s);
       StepParams hp{0.f, 0.f, damping, (double)g->n};
@@ -1116,10 +1147,7 @@ gpr_status run_pagerank(gpr_graph* g, double damping, int32_t iters, gpr_dtype d
         std::chrono::duration<double, std::milli>(std::chrono::steady_clock::now() - t_setup0).count();
     if (st) GPR_CUDA(cudaEventRecord(w->ev_t0, s));
     if (persist) {
-      if (dt == GPR_BF16)
-        run_persist<__nv_bfloat16>(g, w, damping, iters, dst, s);
-      else
-        run_persist<float>(g, w, damping, iters, dst, s);
+      persist_run(g, w, damping, iters, dt, dst, s);
       if (st) GPR_CUDA(cudaEventRecord(w->ev_t1, s));
     } else {
       GPR_CUDA(cudaGraphLaunch(w->exec, s));

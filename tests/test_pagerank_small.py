@@ -118,3 +118,21 @@ def test_lines_of_the_single_launch(n, m, one):
     want = torch.zeros(n, device="cuda")
     want[dst.long()] = m ** -0.5
     assert float((a - want).norm()) <= 1e-5 and float((h - want.roll(1)).norm()) <= 1e-5
+
+
+def test_tuner_times_the_single_launch():
+    # the pull schedule of a small graph is timed as a call runs it: the same time
+    # within a half (the pull kernels take more than twice as long here)
+    import torch
+    n, m = 180_000, 2_500_000
+    gen = torch.Generator(device="cuda").manual_seed(4)
+    src, dst = (torch.randint(0, n, (m,), dtype=torch.int32, device="cuda", generator=gen) for _ in range(2))
+    g = gpr.graph_build(src, dst, n)
+    x = torch.empty(n, dtype=torch.float32, device="cuda")
+    r = gpr.pagerank_tune(g, trial_steps=100)
+    best = min(gpr.pagerank(g, x, iters=100, spmv="pull", stats=True).t_iter_ms for _ in range(5))
+    assert r.pull_ms_per_step * 100 <= 1.5 * best
+    assert r.schedule == gpr.SPMV_PULL and r.ms_per_step == r.pull_ms_per_step
+    before = gpr.lib().gpr_kernel_launches()
+    gpr.pagerank(g, x, iters=100)
+    assert gpr.lib().gpr_kernel_launches() - before == 1
