@@ -315,8 +315,8 @@ gpr_status ppr_batch(const gpr_ppr_job* jobs, int32_t num_jobs, int32_t max_iter
  * (trial_steps in [1, 1000] steps per trial; the jobs' outputs are
  * overwritten) and keeps the fastest for later ppr_batch calls in this
  * process; a class never tuned runs step by step.  The environment variable
- * GPR_PPR_CLUSTER=1|2|4|8 forces one cluster shape for every class.  A
- * column's bits depend on its class's schedule (the order of its sums),
+ * GPR_PPR_CLUSTER=1|2|4|8 forces one cluster shape for every class, 0 the
+ * step-by-step schedule.  A column's bits depend on its class's schedule (the order of its sums),
  * never on the other columns or jobs of a call.
  * Synchronous.  out may be NULL. */
 typedef struct {
@@ -326,6 +326,8 @@ typedef struct {
   int32_t cluster[5];      /* CTAs per cluster of the fastest cluster shape */
   double ms[5];            /* trial time with that shape */
   double ms_cluster8[5];   /* trial time with 8 CTAs per cluster */
+  int32_t kept[5];         /* what later calls run: CTAs per cluster, 0: step by step */
+  double ms_steps[5];      /* trial time of the step-by-step schedule */
 } gpr_ppr_tune_result;
 
 gpr_status ppr_tune(const gpr_ppr_job* jobs, int32_t num_jobs, gpr_dtype dt, int32_t trial_steps,

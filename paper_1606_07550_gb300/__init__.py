@@ -124,7 +124,8 @@ class TuneResult(ctypes.Structure):
 
 class PprTuneResult(ctypes.Structure):
     _fields_ = [("classes", ctypes.c_int32), ("log2n_max", ctypes.c_int32 * 5), ("jobs", ctypes.c_int32 * 5),
-                ("cluster", ctypes.c_int32 * 5), ("ms", ctypes.c_double * 5), ("ms_cluster8", ctypes.c_double * 5)]
+                ("cluster", ctypes.c_int32 * 5), ("ms", ctypes.c_double * 5), ("ms_cluster8", ctypes.c_double * 5),
+                ("kept", ctypes.c_int32 * 5), ("ms_steps", ctypes.c_double * 5)]
 
 
 class Stats(ctypes.Structure):
@@ -443,15 +444,17 @@ def ppr_batch(requests, max_iters: int = 50, tol: float = 0.0, dtype: int = FP32
 
 
 def ppr_tune(requests, dtype: int = FP32, trial_steps: int = 8, stream=None):
-    """Times the cluster shapes of the batched launch for each graph-size
-    class of `requests` (as for ppr_batch; their outputs are overwritten) and
-    keeps the fastest.  Returns one dict per class: log2n_max, jobs, cluster,
-    ms, ms_cluster8."""
+    """Times the cluster shapes and the step-by-step schedule of ppr_batch for
+    each graph-size class of `requests` (as for ppr_batch; their outputs are
+    overwritten) and keeps the fastest.  Returns one dict per class: log2n_max,
+    jobs, cluster and ms (the fastest cluster shape and its time), ms_cluster8,
+    ms_steps (step by step) and kept (the shape that later calls take, 0: step
+    by step)."""
     arr, n_req, keep, _ = _ppr_jobs(requests)
     r = PprTuneResult()
     _check(lib().ppr_tune(arr, n_req, dtype, trial_steps, ctypes.byref(r), _stream_ptr(stream)))
     return [{"log2n_max": r.log2n_max[i], "jobs": r.jobs[i], "cluster": r.cluster[i], "ms": r.ms[i],
-             "ms_cluster8": r.ms_cluster8[i]} for i in range(r.classes)]
+             "ms_cluster8": r.ms_cluster8[i], "ms_steps": r.ms_steps[i], "kept": r.kept[i]} for i in range(r.classes)]
 
 
 class Server:

@@ -40,6 +40,7 @@
 #include <algorithm>
 #include <climits>
 #include <cstdlib>
+#include <cstring>
 #include <map>
 #include <mutex>
 #include <numeric>
@@ -582,12 +583,14 @@ static int class_log2n_max(int k) { return k == kPprClasses - 1 ? 31 : 11 + 2 * 
 static std::mutex g_ppr_tune_mu;
 static std::map<std::pair<int, int>, int> g_ppr_tuned;  // (class, dtype) -> CTAs per cluster
 
-// GPR_PPR_CLUSTER=k (1, 2, 4 or 8) forces the shape of every class.
-static int env_cluster() {
+// GPR_PPR_CLUSTER=k (1, 2, 4 or 8; 0: step by step) forces the schedule of every
+// class; -1: not forced.
+static int env_shape() {
   const char* e = getenv("GPR_PPR_CLUSTER");
-  if (!e) return 0;
+  if (!e) return -1;
+  if (!strcmp(e, "0")) return kStepMajor;
   const int k = atoi(e);
-  return (k == 1 || k == 2 || k == 4 || k == 8) ? k : 0;
+  return (k == 1 || k == 2 || k == 4 || k == 8) ? k : -1;
 }
 
 // Bytes per workspace row (64 columns): the rank state and two contribution
@@ -617,14 +620,15 @@ static void launch_set(PprJob* jobs_dev, const std::vector<int32_t>& order, int3
   ppr_launch(jobs_dev, order_dev, nj, queue, ws, stride, clusters, cluster, dt, s);
 }
 
-// Times each cluster shape on up to kTuneSampleJobs jobs of one class
-// (trial_steps steps from fresh columns) and returns the fastest; ms_out[i]
-// gets candidate i's time.  The trial writes into the jobs' outputs, which
-// the call's real run then overwrites.
+// Times each cluster shape and the step-major schedule on up to kTuneSampleJobs
+// jobs of one class (trial_steps steps from fresh columns) and returns the fastest
+// cluster shape; ms_out[i] gets candidate i's time, ms_out[4] the step-major
+// schedule's.  The trial writes into the jobs' outputs, which the call's real run
+// then overwrites.
 template <typename A>
 static int tune_class(const std::vector<PprJob>& dj, const std::vector<std::vector<PprCol>>& cols,
                       const std::vector<StepRequest>& reqs, const std::vector<int32_t>& members, int32_t n_cap,
-                      gpr_dtype dt, int32_t trial_steps, cudaStream_t s, A alloc, double* ms_out, bool* step_major) {
+                      gpr_dtype dt, int32_t trial_steps, cudaStream_t s, A alloc, double* ms_out) {
   std::vector<int32_t> pick;
   const int32_t step = std::max<int32_t>(1, (int32_t)members.size() / kTuneSampleJobs);
   for (size_t i = 0; i < members.size() && (int32_t)pick.size() < kTuneSampleJobs; i += step) pick.push_back(members[i]);
@@ -672,12 +676,8 @@ static int tune_class(const std::vector<PprJob>& dj, const std::vector<std::vect
         GPR_CUDA(cudaStreamSynchronize(s));
         GPR_CUDA(cudaEventElapsedTime(&ms, e0, e1));
       }
-      if (cl == kStepMajor) {
-        *step_major = ms < best_ms;
-        break;
-      }
       ms_out[ci] = ms;
-      if (ci == 0 || ms < best_ms) {
+      if (cl != kStepMajor && (ci == 0 || ms < best_ms)) {
         best = cl;
         best_ms = ms;
       }
@@ -778,7 +778,7 @@ static gpr_status run_ppr(const gpr_ppr_job* jobs, int32_t num_jobs, int32_t max
     PprJob* jobs_dev = (PprJob*)T((size_t)nj * sizeof(PprJob));
     GPR_CUDA(cudaMemcpyAsync(jobs_dev, dj.data(), (size_t)nj * sizeof(PprJob), cudaMemcpyHostToDevice, s));
     // the shape of each class
-    const int forced = env_cluster();
+    const int forced = env_shape();
     int shape[kPprClasses];
     for (int k = 0; k < kPprClasses; ++k) {
       shape[k] = kDefaultShape[k];
@@ -790,25 +790,28 @@ static gpr_status run_ppr(const gpr_ppr_job* jobs, int32_t num_jobs, int32_t max
         if (it != g_ppr_tuned.end()) shape[k] = it->second;
       }
       if (tune_all) {
-        double ms[4] = {0, 0, 0, 0};
-        bool step_major = false;
-        shape[k] = tune_class(dj, cols, reqs, members[k], ncap[k], dt, std::max(1, trial_steps), s, T, ms, &step_major);
+        double ms[5] = {0, 0, 0, 0, 0}, best_ms = 0.0;
+        const int cluster = tune_class(dj, cols, reqs, members[k], ncap[k], dt, std::max(1, trial_steps), s, T, ms);
+        for (int ci = 0; ci < 4; ++ci)
+          if (kClusterCands[ci] == cluster) best_ms = ms[ci];
+        shape[k] = ms[4] < best_ms ? kStepMajor : cluster;
         {
           std::lock_guard<std::mutex> lk(g_ppr_tune_mu);
-          g_ppr_tuned[key] = step_major ? kStepMajor : shape[k];
+          g_ppr_tuned[key] = shape[k];
         }
         if (tres) {
           const int c = tres->classes++;
           tres->log2n_max[c] = class_log2n_max(k);
           tres->jobs[c] = (int32_t)members[k].size();
-          tres->cluster[c] = shape[k];
-          for (int ci = 0; ci < 4; ++ci) {
-            if (kClusterCands[ci] == shape[k]) tres->ms[c] = ms[ci];
+          tres->cluster[c] = cluster;
+          tres->ms[c] = best_ms;
+          for (int ci = 0; ci < 4; ++ci)
             if (kClusterCands[ci] == 8) tres->ms_cluster8[c] = ms[ci];
-          }
+          tres->kept[c] = shape[k];
+          tres->ms_steps[c] = ms[4];
         }
       }
-      if (forced) shape[k] = forced;
+      if (forced >= 0) shape[k] = forced;
     }
     if (tune_all) {
       GPR_CUDA(cudaStreamSynchronize(s));
