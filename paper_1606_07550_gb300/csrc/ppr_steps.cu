@@ -14,8 +14,8 @@
 // row slot on each.  Lanes hold four columns each (one when W = 1), so a
 // 64-column gather is one 16-byte load per lane and two edges per load.
 //
-// Waves.  The jobs of a width run in waves of up to kWaveBytes of contributions,
-// every job of a wave at the same step.  A launch takes its items job by job, so
+// Waves.  The jobs of a width run in waves of up to kWaveBytes of workspace, every
+// job of a wave at the same step.  A launch takes its items job by job, so
 // the blocks on the GPU at one time gather from few jobs, whose previous
 // contributions L2 (129 MB) and, being written by an earlier launch, the L1s
 // can hold.
@@ -1076,12 +1076,12 @@ __global__ void __launch_bounds__(kStThreads) ppr_out_kernel(const StepJob* __re
 
 static int width_of(int k) { return k <= 1 ? 1 : k <= 4 ? 4 : k <= 16 ? 16 : 64; }
 
-// Contribution buffers of one wave together, at most (a larger job is a wave of
-// its own).  256 batch graphs x 64 columns, 50 steps: 368 ms with waves of
-// 128 MB, 293 ms with 1 GB, 270 ms with one wave of 4.8 GB: a launch's start and
-// end cost more than what waves small enough for L2 save, since a launch takes
-// its items job by job.
-constexpr int64_t kWaveBytes = (int64_t)8 << 30;
+// Workspace of one wave, at most (a larger job is a wave of its own): as much as
+// the cluster schedule's launches take.  256 batch graphs x 64 columns, 50 steps:
+// 368 ms with waves of 192 MB, 293 ms with 1.5 GB, 270 ms with one wave of 7.2 GB: a
+// launch's start and end cost more than what waves small enough for L2 save,
+// since a launch takes its items job by job.
+constexpr int64_t kWaveBytes = (int64_t)16 << 30;
 constexpr int64_t kMinWaveBytes = (int64_t)64 << 20;  // tried down to here when memory is short
 constexpr int64_t kMaxPer = 4;                        // pieces per warp of an item
 
@@ -1164,20 +1164,23 @@ static void run_waves(const std::vector<StepRequest>& reqs, int32_t max_iters, b
     });
     std::vector<Wave> waves;
     std::vector<StepJob> jobs;
-    int64_t ws_bytes = 0, bound_bytes = 0, used = 0, wave_c = 0;
+    int64_t ws_bytes = 0, bound_bytes = 0, used = 0, wave = 0;
     for (int32_t r : order) {
       const gpr_graph* g = reqs[r].graph;
       const int w = width_of(reqs[r].k);
-      const int64_t cells = (int64_t)g->n * w, c_bytes = 2 * cells * tsz;
-      if (waves.empty() || waves.back().w != w || wave_c + c_bytes > wave_bytes) {
+      const int64_t cells = (int64_t)g->n * w;
+      const int64_t chunks = g->m / (kLongDeg / 2);  // a long row's chunks are at least half full
+      const int64_t bytes = cells * (4 + 2 * tsz + (dt == GPR_BF16 ? 4 : 0)) + (int64_t)g->n * 4 +
+                            chunks * (w * 4 + (int64_t)sizeof(LongChunk));
+      if (waves.empty() || waves.back().w != w || wave + bytes > wave_bytes) {
         Wave wv{};
         wv.w = w;
         wv.job0 = (int32_t)jobs.size();
         waves.push_back(wv);
-        used = wave_c = 0;
+        used = wave = 0;
       }
       Wave& wv = waves.back();
-      wave_c += c_bytes;
+      wave += bytes;
       StepJob J{};
       J.col_ptr = g->col_ptr;
       J.row_idx = g->row_idx;
@@ -1207,7 +1210,7 @@ static void run_waves(const std::vector<StepRequest>& reqs, int32_t max_iters, b
       jobs.push_back(J);
       ++wv.jobs;
       wv.work += work(r);
-      wv.chunks += g->m / (kLongDeg / 2);  // a long row's chunks are at least half full
+      wv.chunks += chunks;
     }
     // items: a block of kStWarps x per pieces, so that a step has several
     // blocks for every SM, and few pieces wait on a block's start and end

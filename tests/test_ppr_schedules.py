@@ -51,3 +51,34 @@ def test_forced_schedules_and_their_bits(case, force, dt):
     for k in (1, 3, 9, 40):
         part, (_, rk) = solve(torch, g, seeds[:k], STEPS, dt)
         assert (part == full[:, :k]).all() and (rk == r64[:k]).all()
+
+
+def test_workspace_of_a_batch_is_bounded(force):
+    # 30 jobs of 2^20 nodes, 64 columns in BF16, are 22.5 GB of state: two waves
+    import ctypes
+    import torch
+    cu = ctypes.CDLL("libcuda.so.1")
+    pool, dev, used = ctypes.c_void_p(), ctypes.c_int(), ctypes.c_uint64()
+    used_now, used_high = 7, 8  # CU_MEMPOOL_ATTR_USED_MEM_CURRENT, _HIGH
+
+    def pool_use(attr):
+        assert cu.cuMemPoolGetAttribute(pool, attr, ctypes.byref(used)) == 0
+        return used.value
+
+    n, k, jobs = 1 << 20, 64, 30
+    gen = torch.Generator(device="cuda").manual_seed(2)
+    src, dst = (torch.randint(0, n, (n,), dtype=torch.int32, device="cuda", generator=gen) for _ in range(2))
+    g = gpr.graph_build(src, dst, n)
+    seeds = np.arange(k, dtype=np.int32) * 977
+    x = [torch.zeros((n, k), dtype=torch.float32, device="cuda") for _ in range(jobs)]
+    assert cu.cuCtxGetDevice(ctypes.byref(dev)) == 0 and cu.cuDeviceGetDefaultMemPool(ctypes.byref(pool), dev) == 0
+    force("0")
+    gpr.ppr_batch([(g, seeds, 0.85, x[0])], max_iters=3, dtype=gpr.BF16)
+    alone = x[0].clone()
+    before = pool_use(used_now)
+    zero = ctypes.c_uint64(0)
+    assert cu.cuMemPoolSetAttribute(pool, used_high, ctypes.byref(zero)) == 0
+    gpr.ppr_batch([(g, seeds, 0.85, o) for o in x], max_iters=3, dtype=gpr.BF16)
+    assert pool_use(used_high) - before <= (16 << 30) + (64 << 20)  # and records, items, piece bounds
+    for o in x:
+        assert torch.equal(o, alone)
