@@ -741,7 +741,7 @@ __global__ void __launch_bounds__(kStThreads, 3) ppr_rows_kernel(const StepJob* 
     if (lane < L) {
 #pragma unroll
       for (int v = 0; v < V; ++v) {
-        s_acc[warp][0][c0 + v] += fix60_signed(dsum[v]);
+        s_acc[warp][0][c0 + v] += std::is_same<T, __nv_bfloat16>::value ? fix60_signed(dsum[v]) : fix60(dsum[v]);
         s_acc[warp][1][c0 + v] += fix60(rsum[v]);
       }
     }
