@@ -82,12 +82,13 @@ typedef struct {
 
 typedef struct {
   int32_t iters_run;
-  double residual_l1; /* ||x_k - x_{k-1}||_1 of the last step, FP64 sum of FP32 terms */
-  double mass;        /* sum of x_k, FP64 */
-  double dangling;    /* dangling mass of x_k, FP64 */
+  double residual_l1; /* ||x_k - x_{k-1}||_1 of the last step, summed likewise */
+  double mass;        /* sum of x_k (see pagerank) */
+  double dangling;    /* dangling mass of x_k (the same) */
   double t_setup_ms;  /* host time this call spent making the workspace, the blocked edge
                          layout and the CUDA graph (0 when all were reused) */
-  double t_iter_ms;   /* device time of the iteration loop (CUDA events on `stream`) */
+  double t_iter_ms;   /* device time of the iteration loop (CUDA events on `stream`; with the
+                         output in the single launch of a small graph) */
   int32_t schedule;   /* the step's schedule: GPR_SPMV_PULL or GPR_SPMV_BLOCKED */
 } gpr_stats;
 
@@ -149,12 +150,21 @@ gpr_status graph_load(const char* path, void* stream, gpr_graph** out);
  * "exp_algs", which times 10 iterations):
  *   x_0 = 1/N;   D_k = sum of x_k over nodes with out-degree 0;
  *   x_{k+1}[v] = (1 - d)/N + d (sum_{u -> v} x_k[u] / outdeg(u) + D_k / N)
- * with each step applied to x_k / sum(x_k) (FP64 mass normalisation).
+ * with each step applied to x_k / sum(x_k) (mass and dangling mass summed in
+ * FP64 over FP32 sums of a warp's rows, or as exact sums of multiples of 2^-60 of
+ * them in the single launch below; the step's two coefficients from them in FP64
+ * or 48 bits, then FP32).
  *   damping : d in (0, 1).   iters : >= 0.
  *   dt      : storage of the contribution vector (GPR_FP32 or GPR_BF16).
  *   x_out   : n floats (FP32 even for BF16 storage), indexed by node id;
  *             device memory, or host memory if flags has GPR_PTR_HOST.
  *   st      : optional; filled if non-NULL (this synchronises `stream`).
+ * A graph of fewer than 2^22 edges, and not many more nodes than edges, takes one
+ * launch for the whole iteration (pull schedule, no warm start).  It starts when
+ * it has a place on every SM, so a launch on another stream that holds some of
+ * them holds it up.  Its blocks wait for each other, a bounded time; should a
+ * wait give up (not expected), every rank is NaN, and a call that synchronises
+ * (st, GPR_PTR_HOST) returns GPR_ETIMEOUT.
  * Calls on one graph must not overlap in time (the graph holds the
  * iteration workspace); order them on one stream. */
 gpr_status pagerank(const gpr_graph* g, double damping, int32_t iters, gpr_dtype dt, int flags,
@@ -196,7 +206,8 @@ gpr_status pagerank_tune(const gpr_graph* g, gpr_dtype dt, int32_t trial_steps, 
  * keeps it with the graph.  The products take the pull schedule, or the
  * blocked one (GPR_SPMV_BLOCKED, the default for graphs of 2^22 or more
  * edges; GPR_SPMV_PULL forces the pull schedule), with the vectors
- * L1-normalised between products.  Calls on one graph must not overlap in time (they
+ * L1-normalised between products, or, with the pull schedule of a graph of fewer
+ * edges, scaled by their largest entry.  Calls on one graph must not overlap in time (they
  * share the graph's workspace with pagerank). */
 gpr_status hits(const gpr_graph* g, int32_t iters, float* hub_out, float* auth_out, int flags, void* stream);
 gpr_status eigen_centrality(const gpr_graph* g, int32_t iters, float* x_out, int flags, void* stream);

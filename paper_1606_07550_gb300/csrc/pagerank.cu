@@ -1066,6 +1066,8 @@ static void run_persist(gpr_graph* g, PagerankWork* w, double damping, int32_t i
   A.c[0] = w->c[0];
   A.c[1] = w->c[1];
   A.bar = (unsigned int*)w->ctl;
+  // fault-injection hook for tests: one arrival short, so that the blocks' wait runs out
+  if (getenv("GPR_INJECT_BARRIER_STALL")) GPR_CUDA(cudaMemsetAsync(A.bar, 0xFF, 4, s));
   A.log_row = (double*)(w->ctl + 16);
   A.sums = (unsigned long long*)(w->ctl + 48);
   A.out = dst;

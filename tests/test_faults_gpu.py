@@ -36,3 +36,27 @@ def test_lookback_wait_times_out_and_device_stays_usable():
     ref = oracle.build_csc(50_000, src, dst)
     cp, ri, od = g.export()
     assert (cp == ref.col_ptr).all() and (ri == ref.row_idx).all()
+
+
+def test_pagerank_barrier_wait_runs_out():
+    # with GPR_INJECT_BARRIER_STALL set, the count of arrivals at the single
+    # launch's barrier starts one short: every block's wait gives up
+    import torch
+    n, m = 40_000, 300_000
+    src, dst = gen.rmat_coo(n, m, seed=6)
+    g = gpr.graph_build(torch.from_numpy(src).cuda(), torch.from_numpy(dst).cuda(), n)
+    x, host = torch.empty(n, device="cuda"), np.empty(n, np.float32)
+    gpr.pagerank(g, x, iters=20)
+    want = x.clone()
+    os.environ["GPR_INJECT_BARRIER_STALL"] = "1"
+    try:
+        gpr.pagerank(g, x, iters=20)  # does not synchronise: NaN ranks
+        assert bool(torch.isnan(x).all())
+        for out, stats in ((x, True), (host, False)):
+            with pytest.raises(gpr.GprError) as ei:
+                gpr.pagerank(g, out, iters=20, stats=stats)
+            assert ei.value.status == gpr.ETIMEOUT
+    finally:
+        os.environ.pop("GPR_INJECT_BARRIER_STALL", None)
+    gpr.pagerank(g, x, iters=20)
+    assert torch.equal(x, want)
