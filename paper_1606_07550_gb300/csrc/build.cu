@@ -434,12 +434,11 @@ static const Sweep kSweep8[8] = {sweep<kManyThreads, 8, 0>(),  sweep<kManyThread
                                  sweep<kManyThreads, 8, 32>(), sweep<kManyThreads, 8, 40>(), sweep<kManyThreads, 8, 48>(), sweep<kManyThreads, 8, 56>()};
 static const Sweep kSweep8Any = sweep<kManyThreads, 8, -1>();
 static const Sweep kSweep9 = sweep<kManyThreads, 9, -1>();
-// Sorts of up to kFewTiles tiles of 4,096 keys: a tile an SM, where larger
-// tiles would leave SMs idle.  With the line at 608 tiles a build of 1.5 M edges
+// Sorts of up to one tile of 4,096 keys an SM (152), where larger tiles would
+// leave SMs idle.  With the line at 608 tiles a build of 1.5 M edges
 // takes 371 us instead of 353 and one of 2 M 435 instead of 386.
 static const Sweep kSweep8Few = sweep<256, 8, -1, 16>();
 static const Sweep kSweep9Few = sweep<256, 9, -1, 16>();
-constexpr int64_t kFewTiles = 152;
 
 // The largest shared-memory carve-out and the blocks' shared memory, once a device.
 static void sweep_attributes() {
@@ -465,7 +464,7 @@ uint64_t* radix_sort_u64(uint64_t* keys, uint64_t* alt, int64_t n, int bits, cud
   const DigitPlan dp = digit_plan(bits, low);
   const int passes = dp.passes;
   if (n <= 1 || passes == 0) return keys;
-  const bool few = n <= kFewTiles * kTile;
+  const bool few = n <= (int64_t)num_sms() * kTile;
   const int64_t tile_keys = (few ? 256 : kManyThreads) * kItems, tiles = (n + tile_keys - 1) / tile_keys;
   int radix = 0;
   for (int p = 0; p < passes; ++p) radix = std::max(radix, 1 << dp.width[p]);

@@ -568,7 +568,6 @@ constexpr int kPprClasses = 5;
 constexpr int kClusterCands[] = {1, 2, 4, 8};
 constexpr int kDefaultCluster = 8;
 constexpr int kStepMajor = 0;  // a class's "shape" when its jobs run step by step over the whole GPU (ppr_steps.cu)
-constexpr int kDefaultShape[kPprClasses] = {kStepMajor, kStepMajor, kStepMajor, kStepMajor, kStepMajor};
 constexpr int32_t kTuneSampleJobs = 64;
 constexpr int64_t kWorkspaceBudget = (int64_t)16 << 30;  // per launch: clusters x stride at most
 
@@ -781,7 +780,7 @@ static gpr_status run_ppr(const gpr_ppr_job* jobs, int32_t num_jobs, int32_t max
     const int forced = env_shape();
     int shape[kPprClasses];
     for (int k = 0; k < kPprClasses; ++k) {
-      shape[k] = kDefaultShape[k];
+      shape[k] = kStepMajor;
       if (members[k].empty()) continue;
       const std::pair<int, int> key(k, (int)dt);
       {
