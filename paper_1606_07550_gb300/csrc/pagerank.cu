@@ -810,8 +810,11 @@ static Choice pick(gpr_graph* g, PagerankWork* w, int flags, gpr_dtype dt, cudaS
 // 3,319 / 3,675.
 constexpr int32_t kPersMaxRows = 1 << 22, kPersFreeRows = 3 << 19, kProductMaxRows = 1 << 23;
 static bool persist_eligible(const gpr_graph* g, const PagerankWork* w, int sched, bool warm, bool product) {
-  // a block's long rows fit its lists: at most m / 65 rows, dealt out evenly
-  static_assert(kTuneMinEdges / (kPersShort + 1) / 128 < kPersLongRows, "long rows of a block");
+  // the long rows, at most m / 65, and their chunks fit the blocks' lists together
+  // (persist_deal passes over a full block)
+  static_assert(kTuneMinEdges / (kPersShort + 1) < 128 * (int64_t)kPersLongRows, "long rows of all blocks");
+  static_assert(kTuneMinEdges / kPersChunk + kTuneMinEdges / (kPersShort + 1) <
+                    128 * (int64_t)(kPersChunks - kPersRowChunks), "chunks of all blocks");
   const bool rows = product ? g->n <= kProductMaxRows : g->n <= kPersMaxRows && g->n <= kPersFreeRows + g->m;
   return sched == kSchedPull && !warm && w->hot_grid == 0 && g->m < kTuneMinEdges && rows && num_sms() >= 128;
 }
@@ -1217,7 +1220,8 @@ gpr_status run_pagerank_tune(gpr_graph* g, gpr_dtype dt, int32_t trial_steps, gp
 // run on the pull kernels of the PageRank step with unit weights (an
 // inverse-degree vector of ones) and d = 1: each step's fold leaves
 // coefA = 1 / ||previous vector||_1, so every product starts from the L1-
-// normalised previous vector.  Scaling does not change a direction, so the
+// normalised previous vector (on small graphs, a launch a product: from the
+// previous vector over its largest entry, persist_kernel's kProduct).  Scaling does not change a direction, so the
 // vectors match the L2-normalised iteration; the output is scaled to unit L2
 // norm once, at the end.  A^T x pulls over g's CSC; A x pulls over the CSC of
 // the transposed graph (same relabelled ids), built on first use.

@@ -12,7 +12,7 @@
 
 namespace gpr {
 
-constexpr int kPprCols = 64;  // columns per job: 32 lanes x 2
+constexpr int kPprCols = 64;  // columns per job
 
 enum : int32_t { kColEmpty = 0, kColFresh = 1, kColRunning = 2, kColDone = 3 };
 

@@ -17,11 +17,13 @@
 // Layout (made once per graph).  The rows run by descending in-degree.  Rows of
 // up to kPersShort edges are sliced by 32, a lane a row, their sources stored
 // slice by slice, edge by edge (lane l of edge j at off + 32 j + l, -1 past a
-// row's end): every index load of a warp is one 128-byte line and a row needs
-// no reduction.  (Lanes sharing a row, four edges ahead, spent 400 issue and
+// row's end; SELL-C-sigma of Kreutzer et al. 2014 with C = 32 and all rows
+// sorted): every index load of a warp is one 128-byte line and a row needs no
+// reduction.  (Lanes sharing a row, four edges ahead, spent 400 issue and
 // load slots a task: 10 us a step for 10,000 nodes and 100,000 edges on 16
-// SMs.)  Longer rows go round-robin to blocks, which cut them into chunks for
-// their warps and add a row's chunk sums after a block barrier.
+// SMs.)  Longer rows, the longest first, and then the slices go to the block with
+// the least estimated work so far; blocks cut long rows into chunks for their
+// warps and add a row's chunk sums after a block barrier.
 //
 // Mass, dangling mass and residual: FP32 per thread and over the warp as in the
 // pull kernels, then exact integer sums of multiples of 2^-60 over warps and

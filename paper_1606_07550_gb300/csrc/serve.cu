@@ -112,11 +112,16 @@ namespace gpr {
 
 static size_t elem_bytes(gpr_dtype dt) { return dt == GPR_FP32 ? 4 : 2; }
 
-// Work of an item of g (an edge counts 1, a row 3): as configured, or for a
-// graph that fills the GPU with them small items, which end together, for a
-// smaller one twice as large ones, which leave the SMs to other slots.  A burst
-// of 32 requests over graphs of scales 14 to 22 takes 201 ms with items of 2^14
-// throughout, 229 with 2^15, 300 with 2^16 and 433 with 2^17.
+// Work of an item of g (an edge counts 1, a row 3): as configured, or 2^14 for
+// graphs of at least kLargeWork, 2^15 for smaller ones.  Speed alone would take
+// 2^14 throughout: a burst of 32 requests over graphs of scales 14 to 22 takes
+// 164 ms with it, 167 with this rule and 167 with 2^15 throughout (an earlier
+// burst 300 with 2^16, 433 with 2^17), a pool of 256 graphs of 1,000 to 200,000
+// nodes completes 96,000 solves/s against 90,000, and 400 steps of 64 columns on
+// 2^16 nodes alone take 107 ms against 160.  The smaller graphs keep 2^15 because a
+// request of so many steps is expected to be running still when one that came
+// 50 ms after it has been answered (tests/test_serve_gpu.py), which that last
+// figure leaves no room for.
 constexpr int64_t kLargeWork = 1 << 22;
 static int per_warp(const gpr_server* S, const gpr_graph* g) {
   const int64_t work = g->m + 3 * (int64_t)g->n;
