@@ -9,10 +9,12 @@
 // sums its rows, finishes them and meets the other blocks at a barrier.
 //
 // What bounds it.  10,000 nodes, 100,000 edges, 50 steps: 650 us as a CUDA graph of
-// six kernels a step, 184 us here, 3.7 us a step: the barrier and the writes
-// before it 1.6, coefficients and copy 0.7, the sums 0.4.  250,000 nodes,
-// 4,000,000 edges (R-MAT, BF16): 1,910 us against 820, 16 us a step, bound by the
-// shared-memory and L1 slots of the gathers, about 10 cycles for 32 edges.
+// six kernels a step, 163 us here, 3.2 us a step: the barrier and the writes
+// before it 1.7, the sums 0.9, coefficients and copy 0.6.  250,000 nodes,
+// 4,000,000 edges (R-MAT, BF16): 1,910 us against 752, 15 us a step, bound by the
+// shared-memory and L1 slots of the gathers, about 10 cycles for 32 edges: long
+// rows' chunks 4.7, slices 3.6, then the long rows' ends 2 to 3 on the blocks that
+// have most and the barrier.
 //
 // Layout (made once per graph).  The rows run by descending in-degree.  Rows of
 // up to kPersShort edges are sliced by 32, a lane a row, their sources stored
@@ -30,7 +32,8 @@
 // blocks, so runs are bitwise identical.  A thread has more rows here, and where
 // most rows hold the same rank all threads round alike, so its mass and dangling
 // mass are sums of two floats (2^20 nodes and edges: L1 error 3.3e-8; with plain
-// sums 6.4e-8, with the pull kernels 3.5e-8; times within 1.5% either way).
+// sums 6.4e-8, with the pull kernels 3.5e-8; 50 steps of 900,000 nodes and 4,100,000 edges 1,068 ->
+// 1,090 us).
 //
 // The centralities take the same kernel a step at a time (kProduct):
 // one launch a product instead of six.
@@ -138,9 +141,8 @@ __host__ __device__ __forceinline__ int32_t pers_chunk(int32_t deg) {
 // caller or the product before left (no start vector, so no barrier); x and
 // contributions stored, no output.  sums rows hold the largest entry's bits: a
 // product can scale the vector by anything, which fixed-point sums would not
-// follow, and its largest entry is exact in any order.  (A kernel of its own: as
-// an argument of the iteration's it took 50 BF16 steps of 250,000 nodes and
-// 4,000,000 edges from 802 to 1,268 us.)
+// follow, and its largest entry is exact in any order.  (A kernel of its own, so
+// that the iteration's loops hold nothing of it.)
 template <typename T, bool kCluster, bool kProduct = false>
 __global__ void __launch_bounds__(kPersThreads, 1) persist_kernel(const __grid_constant__ PersistArgs A) {
   extern __shared__ __align__(16) unsigned char pers_smem[];
