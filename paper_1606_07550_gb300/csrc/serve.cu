@@ -641,6 +641,9 @@ gpr_status serve_fetch(gpr_server* S, uint64_t ticket, float* dst, int flags) {
     bytes = (size_t)it->second.result_bytes;
   }
   cudaError_t e = cudaMemcpy(dst, src, bytes, (flags & GPR_PTR_HOST) ? cudaMemcpyDeviceToHost : cudaMemcpyDeviceToDevice);
+  // (the host does not wait for a copy inside device memory; serve_release may give
+  // the source to the next request, on the server's stream)
+  if (e == cudaSuccess && !(flags & GPR_PTR_HOST)) e = cudaStreamSynchronize(cudaStreamLegacy);
   if (e != cudaSuccess) {
     set_error("serve_fetch: %s", cudaGetErrorString(e));
     return GPR_ECUDA;

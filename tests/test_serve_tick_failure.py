@@ -62,3 +62,27 @@ def test_requests_after_a_failed_tick(dt, err):
     st = srv.stats()
     assert st["completed"] == 3 and st["failed"] == 1 and st["device_bytes_in_use"] == pool_bytes
     srv.close()
+
+
+def test_fetch_to_device_memory_waits_for_its_copy():
+    # the copy goes behind what the default stream holds, here about a second of
+    # waiting: after it the result may be released and its memory used again
+    import time
+    import torch
+    src, dst = gen.rmat_coo(3000, 40_000, seed=61)
+    g = gpr.graph_build(src, dst, 3000)
+    srv = gpr.Server([g], budget_bytes=4 << 30)
+    t = srv.submit(0, [5], max_iters=20)
+    r = wait(srv, t)
+    out = torch.zeros(r.n, device="cuda")
+    torch.cuda.synchronize()
+    start, end = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
+    start.record()
+    torch.cuda._sleep(1_000_000_000)
+    end.record()
+    t0 = time.perf_counter()
+    srv.fetch(t, out)
+    waited = time.perf_counter() - t0
+    assert end.query() and waited >= 0.5e-3 * start.elapsed_time(end)
+    srv.release(t)
+    srv.close()
