@@ -310,7 +310,7 @@ typedef struct {
 /* jobs: host array of num_jobs >= 0 jobs (graphs may repeat).  max_iters in
  * [0, 2^20]; tol >= 0 (0: run exactly max_iters steps).  dt: storage of the
  * gathered contributions (the rank state and accumulation stay FP32).
- * The workspace is taken for the call: up to 16 GB for as many jobs as that
+ * The workspace is taken for the call: up to 8 GB for as many jobs as that
  * holds, or what one larger job needs; less where that cannot be allocated.
  * Synchronises `stream`.  Errors: GPR_EINVAL for a bad argument (nothing
  * launched), GPR_ENOMEM, GPR_ECUDA. */

@@ -1076,12 +1076,13 @@ __global__ void __launch_bounds__(kStThreads) ppr_out_kernel(const StepJob* __re
 
 static int width_of(int k) { return k <= 1 ? 1 : k <= 4 ? 4 : k <= 16 ? 16 : 64; }
 
-// Workspace of one wave, at most (a larger job is a wave of its own): as much as
-// the cluster schedule's launches take.  256 batch graphs x 64 columns, 50 steps:
-// 368 ms with waves of 192 MB, 293 ms with 1.5 GB, 270 ms with one wave of 7.2 GB: a
-// launch's start and end cost more than what waves small enough for L2 save,
-// since a launch takes its items job by job.
-constexpr int64_t kWaveBytes = (int64_t)16 << 30;
+// Workspace of one wave, at most (a larger job is a wave of its own).  256 batch
+// graphs x 64 columns, 50 steps: 368 ms with waves of 192 MB, 293 ms with 1.5 GB,
+// 270 ms with one wave of 7.2 GB: a launch's start and end cost more than what
+// waves small enough for L2 save, since a launch takes its items job by job.  Above
+// that nothing is gained: 4,096 graphs in FP32 / BF16 3.99 / 4.17 s with 8 GB, 4.01 /
+// 4.28 with 12, 4.04 / 4.38 with 16.
+constexpr int64_t kWaveBytes = (int64_t)8 << 30;
 constexpr int64_t kMinWaveBytes = (int64_t)64 << 20;  // tried down to here when memory is short
 constexpr int64_t kMaxPer = 4;                        // pieces per warp of an item
 

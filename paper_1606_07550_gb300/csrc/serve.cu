@@ -115,7 +115,7 @@ static size_t elem_bytes(gpr_dtype dt) { return dt == GPR_FP32 ? 4 : 2; }
 // Work of an item of g (an edge counts 1, a row 3): as configured, or 2^14 for
 // graphs of at least kLargeWork, 2^15 for smaller ones.  Speed alone would take
 // 2^14 throughout: a burst of 32 requests over graphs of scales 14 to 22 takes
-// 164 ms with it, 167 with this rule and 167 with 2^15 throughout (an earlier
+// 164 ms with it, 166 with this rule and 168 with 2^15 throughout (an earlier
 // burst 300 with 2^16, 433 with 2^17), a pool of 256 graphs of 1,000 to 200,000
 // nodes completes 96,000 solves/s against 90,000, and 400 steps of 64 columns on
 // 2^16 nodes alone take 107 ms against 160.  The smaller graphs keep 2^15 because a
