@@ -136,3 +136,20 @@ def test_tuner_times_the_single_launch():
     before = gpr.lib().gpr_kernel_launches()
     gpr.pagerank(g, x, iters=100)
     assert gpr.lib().gpr_kernel_launches() - before == 1
+
+
+def test_hub_of_equal_contributions():
+    # every node points at node 0, which points back: one row of 23,074 equal
+    # numbers, 64 chunks of 361 edges.  A chunk's sum rounds at most 3 times in a
+    # lane's group, twice over its groups and 5 times over the warp, the chunks' 3 times
+    # in an eight and 8 times over the eights, half an ulp of 2^-24 each, all the
+    # same way: 0.85 * 21 * 2^-25; the start vector, the coefficients and the other
+    # nodes (0.15 of the mass) round by 1.1e-7 together
+    import torch
+    n = 23_075
+    o = np.arange(1, n, dtype=np.int32)
+    z = np.zeros(n - 1, np.int32)
+    src, dst = np.concatenate([o, z]), np.concatenate([z, o])
+    g = gpr.graph_build(src, dst, n)
+    x, _ = run(torch, g, 1, gpr.FP32)
+    assert l1(x, oracle.pagerank(oracle.build_csc(n, src, dst), 0.85, 1)) <= 0.85 * 21 * 2.0 ** -25 + 1.1e-7

@@ -117,3 +117,24 @@ def test_bf16_rows_below_zero(k):
     gpr.ppr_batch([(g, seeds, 0.999, x)], max_iters=30, dtype=gpr.BF16)
     for j in range(min(k, 2)):
         assert l1(x[:, j].cpu().numpy(), oracle.ppr(ref, int(seeds[j]), 0.999, 30)[0]) <= 0.12
+
+
+@pytest.mark.gpu
+@pytest.mark.parametrize("k", [1, 4, 16, 64])
+def test_hub_of_equal_contributions(k):
+    # 130,000 nodes point at node 0, which points back: after two steps from node 0
+    # its row sums as many equal numbers, 0.85 of the mass, in 508 chunks of 256 edges.
+    # A slot rounds at most 8 times, the slots of a block twice, four blocks, the two
+    # halves, 7 additions of an eight and 64 over the eights, half an ulp of 2^-24 each,
+    # all the same way: 0.85 * 0.85 * 86 * 2^-25; the other roundings are 2.5e-7 together
+    import torch
+    n = 130_001
+    o = np.arange(1, n, dtype=np.int32)
+    z = np.zeros(n - 1, np.int32)
+    src, dst = np.concatenate([o, z]), np.concatenate([z, o])
+    g, ref = gpr.graph_build(src, dst, n), oracle.build_csc(n, src, dst)
+    x = torch.zeros((n, k), dtype=torch.float32, device="cuda")
+    gpr.ppr_batch([(g, np.zeros(k, np.int32), 0.85, x)], max_iters=2)
+    want = oracle.ppr(ref, 0, 0.85, 2)[0]
+    for j in {0, k - 1}:
+        assert l1(x[:, j].cpu().numpy(), want) <= 0.85 * 0.85 * 86 * 2.0 ** -25 + 2.5e-7
