@@ -525,7 +525,7 @@ def ppr_bytes_per_step(n, m, dt_name, cols=64):
 def run_batched(args, world, rank, local):
     """Config: 4,096 R-MAT graphs (n log-uniform in [1e3, 2e5], mean out-degree
     uniform in [4, 32]), 64 personalised-PageRank seeds each, damping 0.85,
-    50 steps, one persistent launch per storage type.  Under torchrun the
+    50 steps, one ppr_batch call per storage type.  Under torchrun the
     graphs are shared out (graph g on rank g % world, no data-path
     collective); value = all ranks' solves over the slowest rank's time.
     Baselines on the same GPU: one solve per call (ppr_batch with one seed)
@@ -653,7 +653,7 @@ def run_batched(args, world, rank, local):
         "config": {"workload": "batched-ppr-4096x64", "graphs": len(specs_all), "seeds_per_graph": 64,
                    "iters": iters, "damping": 0.85, "sum_n": sum_n, "sum_m": sum_m,
                    "sum_m_raw": sum(sp.m for sp in specs_all),
-                   "step": "one ppr_batch call: every column of every graph (of this rank), one persistent launch",
+                   "step": "one ppr_batch call: every column of every graph (of this rank), step by step over the GPU or on clusters, as tuned",
                    "parallelism": f"graphs sharded over {world} rank(s), g % world",
                    "l2": "per-job state 0.3-77 MB; the batch's working set far above L2"},
         "by_dtype": res,

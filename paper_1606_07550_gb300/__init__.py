@@ -432,7 +432,7 @@ def _ppr_jobs(requests):
 
 
 def ppr_batch(requests, max_iters: int = 50, tol: float = 0.0, dtype: int = FP32, stream=None):
-    """Personalised PageRank for many (graph, seeds) requests in one launch.
+    """Personalised PageRank for many (graph, seeds) requests in one call.
 
     requests: list of (graph, seeds, damping, out) with seeds an int sequence,
     damping a float or a per-seed sequence, out a CUDA float32 tensor of shape
